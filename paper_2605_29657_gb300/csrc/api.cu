@@ -760,7 +760,6 @@ int occam_threshold(const occam_batch* batch, const float* s, const float* ref, 
   WsLayout L;
   OCCAM_TRY(check_ws(batch, 1, 1, workspace, workspace_bytes, &L));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
   if (count_vis) OCCAM_CUDA(cudaMemsetAsync(count_vis, 0, batch->B * 4, st));
   ThresholdParams p;
   p.bt = dev_batch(batch);
@@ -770,10 +769,10 @@ int occam_threshold(const occam_batch* batch, const float* s, const float* ref, 
   p.lambda = lambda;
   p.prev_keep = prev_keep;
   p.keep_registers = keep_registers;
-  p.role = at<uint8_t>(workspace, L.role);
   p.keep = keep;
   p.count_vis = count_vis;
-  threshold_kernel<<<(unsigned)cdiv(batch->total_rows, 256), 256, 0, st>>>(p);
+  const dim3 grid((unsigned)batch->S_tot, (unsigned)std::min<int64_t>(cdiv(batch->max_seg_rows, kThrRows), 256));
+  threshold_kernel<<<grid, 256, 0, st>>>(p);
   count_launch();
   return cuda_ok();
 }
@@ -788,11 +787,13 @@ int occam_mean_reference(const occam_batch* batch, const float* s, int32_t ref_s
   WsLayout L;
   OCCAM_TRY(check_ws(batch, 1, 1, workspace, workspace_bytes, &L));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
+  // units larger than the kernel's register bits: row roles in the workspace
+  const bool roles = (ref_scope == OCCAM_REF_SEGMENT ? batch->max_seg_rows : batch->max_sample_rows) > kRegBitRows;
+  if (roles) OCCAM_TRY(mark_roles(batch, L, workspace, st));
   MeanRefParams p;
   p.bt = dev_batch(batch);
   p.s = s;
-  p.role = at<uint8_t>(workspace, L.role);
+  p.role = roles ? at<uint8_t>(workspace, L.role) : nullptr;
   p.prev_keep = prev_keep;
   p.scope = ref_scope;
   p.ref = ref;
@@ -830,18 +831,19 @@ int occam_budget_keep(const occam_batch* batch, const float* s, const uint8_t* p
   WsLayout L;
   OCCAM_TRY(check_ws(batch, 1, 1, workspace, workspace_bytes, &L));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
+  // samples larger than the kernel's register bits: row roles in the workspace
+  const bool roles = batch->max_sample_rows > kRegBitRows;
+  if (roles) OCCAM_TRY(mark_roles(batch, L, workspace, st));
   BudgetParams p;
   p.bt = dev_batch(batch);
   p.s = s;
-  p.role = at<uint8_t>(workspace, L.role);
+  p.role = roles ? at<uint8_t>(workspace, L.role) : nullptr;
   p.prev_keep = prev_keep;
   p.budget = budget;
   p.keep_registers = keep_registers;
   p.keep = keep;
   p.count_vis = count_vis;
-  budget_keep_kernel<<<batch->B, 1024, 0, st>>>(p);
-  count_launch();
+  if (launch_budget_keep(p, batch->max_sample_rows, st) != 0) return OCCAM_ERR_CUDA;
   return cuda_ok();
 }
 
@@ -983,9 +985,7 @@ static int prune_impl(const occam_prune_args* args, const occam_prune_out* out, 
     bp.keep_registers = args->keep_registers;
     bp.keep = out->keep2;
     bp.count_vis = nullptr;
-    budget_keep_kernel<<<b->B, 1024, 0, st>>>(bp);
-    count_launch();
-    OCCAM_CUDA(cudaGetLastError());
+    if (launch_budget_keep(bp, b->max_sample_rows, st) != 0) return OCCAM_ERR_CUDA;
     // no Stage-II threshold under the budget rule: no near-threshold rows
     if (out->near2) OCCAM_CUDA(cudaMemsetAsync(out->near2, 0, b->total_rows, st));
     return launch_compact(b, L, ws, 0, out->keep2, nullptr, nullptr, args->keep_registers, nullptr, args->n_tensors,

@@ -160,6 +160,26 @@ __device__ __forceinline__ int upper_interval(const T* off, int n, int64_t x) {
   return lo;
 }
 
+// Register flags of the rows [lo, lo + n), n <= 32 * words, as bits in shared
+// memory: row lo + i is bit i. reg_idx[ra .. rb) lists the registers that may
+// lie among them. A kernel that looks at whole segments or samples marks its
+// own rows this way, without the row-role bytes in global memory (a memset
+// and a scatter ahead of it, 2-3 us each, as long as the work itself).
+// Contains __syncthreads before and after the marking.
+constexpr int kRegBitWords = 2048;
+constexpr int kRegBitRows = 32 * kRegBitWords;
+__device__ __forceinline__ void mark_register_bits(uint32_t* bits, int64_t lo, int n, const int32_t* reg_idx, int ra,
+                                                   int rb) {
+  for (int i = threadIdx.x; i < (n + 31) / 32; i += blockDim.x) bits[i] = 0;
+  __syncthreads();
+  for (int i = ra + threadIdx.x; i < rb; i += blockDim.x) {
+    const int64_t r = reg_idx[i] - lo;
+    if (r >= 0 && r < n) atomicOr(&bits[r >> 5], 1u << (r & 31));
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ bool test_bit(const uint32_t* bits, int i) { return (bits[i >> 5] >> (i & 31)) & 1u; }
+
 // First index i in [0, n] with off[i] >= x (off ascending, [n+1] entries).
 template <typename T>
 __device__ __forceinline__ int lower_bound_off(const T* off, int n, int64_t x) {

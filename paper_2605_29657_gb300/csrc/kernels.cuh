@@ -85,7 +85,6 @@ struct ThresholdParams {
   float lambda;
   const uint8_t* prev_keep;
   int keep_registers;
-  const uint8_t* role;
   uint8_t* keep;
   int32_t* count_vis;
 };
@@ -253,7 +252,7 @@ constexpr int kL2SelBytes = 32 * 1024;  // workspace scratch of the selection
 struct MeanRefParams {
   BatchDev bt;
   const float* s;
-  const uint8_t* role;
+  const uint8_t* role;       // nullable: the kernel marks the unit's registers itself (units of <= kRegBitRows rows)
   const uint8_t* prev_keep;  // nullable
   int scope;                 // OCCAM_REF_SEGMENT or OCCAM_REF_SAMPLE
   float* ref;                // [units]
@@ -266,7 +265,7 @@ struct MeanRefParams {
 struct BudgetParams {
   BatchDev bt;
   const float* s;
-  const uint8_t* role;
+  const uint8_t* role;       // nullable, as in MeanRefParams
   const uint8_t* prev_keep;  // nullable
   const int32_t* budget;     // [B]
   int keep_registers;
@@ -308,6 +307,7 @@ __global__ void stage1_finalize_kernel(Stage1FinalizeParams p);
 void launch_mutual_tc(const MutualTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mq1,
                       const CUtensorMap& mk1, int sms, cudaStream_t st);
 __global__ void roles_scatter_kernel(BatchDev bt, uint8_t* role);
+constexpr int kThrRows = 2048;  // rows of a segment a threshold CTA takes at a time
 __global__ void threshold_kernel(ThresholdParams p);
 
 // stage2.cu
@@ -337,7 +337,7 @@ __global__ void registers_kernel(RegistersParams p);
 
 // rules.cu
 __global__ void mean_ref_kernel(MeanRefParams p);
-__global__ void budget_keep_kernel(BudgetParams p);
+int launch_budget_keep(const BudgetParams& p, int64_t max_sample_rows, cudaStream_t st);
 __global__ void pool_scores_kernel(const float* s_in, int64_t rows_out, int group, int mode, float* s_out);
 __global__ void gather_kernel(GatherParams p);
 __global__ void offsets_fix_kernel(ScanParams p);

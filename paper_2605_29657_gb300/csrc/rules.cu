@@ -31,13 +31,20 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 __global__ void __launch_bounds__(256) mean_ref_kernel(MeanRefParams p) {
   __shared__ double wsum[8];
   __shared__ int wcnt[8];
+  __shared__ uint32_t bits[kRegBitWords];
   const int u = blockIdx.x, tid = threadIdx.x;
   const int64_t lo = p.scope == OCCAM_REF_SEGMENT ? p.bt.seg_off[u] : p.bt.row_off[u];
   const int64_t hi = p.scope == OCCAM_REF_SEGMENT ? p.bt.seg_off[u + 1] : p.bt.row_off[u + 1];
+  if (!p.role) {
+    const int sa = p.scope == OCCAM_REF_SEGMENT ? u : p.bt.seg_first[u];
+    const int sz = p.scope == OCCAM_REF_SEGMENT ? u + 1 : p.bt.seg_first[u + 1];
+    mark_register_bits(bits, lo, (int)min(hi - lo, (int64_t)kRegBitRows), p.bt.reg_idx, p.bt.reg_off[sa],
+                       p.bt.reg_off[sz]);
+  }
   double acc = 0.0;
   int cnt = 0;
   for (int64_t r = lo + tid; r < hi; r += blockDim.x) {
-    if (p.role[r] == 0 && (!p.prev_keep || p.prev_keep[r] != 0)) {
+    if (!(p.role ? p.role[r] != 0 : test_bit(bits, (int)(r - lo))) && (!p.prev_keep || p.prev_keep[r] != 0)) {
       acc += (double)p.s[r];
       ++cnt;
     }
@@ -70,104 +77,169 @@ __device__ __forceinline__ uint32_t order_key(float v) {
 }
 
 // One CTA of 1,024 threads per sample.
-//   1. n = the sample's candidate count; K = clamp(budget[b], 0, n).
-//   2. If 0 < K < n: the K-th largest candidate key t, most significant byte
-//      first (per byte a 256-bin histogram of the keys that match the bytes
-//      chosen so far, one histogram per warp, summed; then the bucket where
-//      the running count from the top reaches K). need = how many keys equal
-//      to t are kept = K - #(keys > t).
-//   3. Each thread takes a contiguous run of the sample's rows: keys above t
-//      are kept; keys equal to t are ranked in row order by a block scan and
-//      the first `need` of them kept. Register rows get keep_registers.
+//   1. Candidate keys (STAGED: once from global memory into shared memory,
+//      with the candidates and registers as bits; else read again by every
+//      pass) and the histogram of their top 11 bits; n = the candidate count,
+//      K = clamp(budget[b], 0, n).
+//   2. If 0 < K < n: the K-th largest candidate key t, eleven bits at a time
+//      (bits 31-21, 20-10, 9-0): a block scan over the 2,048 buckets finds
+//      the one where the running count from the top reaches K. need = how
+//      many keys equal to t are kept = K - #(keys > t).
+//   3. Keys above t are kept, and those equal to t if all of them are
+//      needed; else they are ranked in row order (each thread a contiguous
+//      run of rows, a block scan) and the first `need` kept. Register rows
+//      get keep_registers.
+// The chain of passes bounds it. With four 8-bit passes over global memory
+// and a serial search of each histogram a sample of 2,900 rows took 30 us.
+template <bool STAGED>
 __global__ void __launch_bounds__(1024) budget_keep_kernel(BudgetParams p) {
-  __shared__ uint32_t hist[32][256];
-  __shared__ uint32_t tot[256];
+  extern __shared__ uint32_t keys[];  // STAGED: the sample's keys
+  __shared__ uint32_t hist[2048];
+  __shared__ uint32_t regs[kRegBitWords], cands[STAGED ? kRegBitWords : 1];
   __shared__ uint32_t s_prefix, s_k;
-  __shared__ int s_cnt;
   __shared__ int tmp[40];
-  const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5;
-  const int64_t lo = p.bt.row_off[b], hi = p.bt.row_off[b + 1];
-  auto cand = [&](int64_t r) { return p.role[r] == 0 && (!p.prev_keep || p.prev_keep[r] != 0); };
-  if (tid == 0) s_cnt = 0;
-  __syncthreads();
-  int c = 0;
-  for (int64_t r = lo + tid; r < hi; r += blockDim.x) c += cand(r) ? 1 : 0;
-  c = warp_sum_i(c);
-  if ((tid & 31) == 0) atomicAdd(&s_cnt, c);
-  __syncthreads();
-  const int n = s_cnt;
-  const int K = min(max(p.budget[b], 0), n);
-  // t = 0 with need = n keeps every candidate (every key is >= 0)
-  uint32_t t = 0;
-  int need = n;
-  if (K == 0) {
-    t = 0xffffffffu;
-    need = 0;
-  } else if (K < n) {
-    if (tid == 0) {
-      s_prefix = 0;
-      s_k = (uint32_t)K;
-    }
-    uint32_t mask = 0;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = tid; i < 32 * 256; i += blockDim.x) (&hist[0][0])[i] = 0;
-      __syncthreads();
-      const uint32_t prefix = s_prefix;
-      for (int64_t r = lo + tid; r < hi; r += blockDim.x) {
-        if (!cand(r)) continue;
-        const uint32_t key = order_key(p.s[r]);
-        if ((key & mask) == prefix) atomicAdd(&hist[warp][(key >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      if (tid < 256) {
-        uint32_t s = 0;
-        for (int w = 0; w < 32; ++w) s += hist[w][tid];
-        tot[tid] = s;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        uint32_t k = s_k, cum = 0;
-        int d = 255;
-        for (; d > 0; --d) {
-          if (cum + tot[d] >= k) break;
-          cum += tot[d];
-        }
-        s_k = k - cum;
-        s_prefix = prefix | ((uint32_t)d << shift);
-      }
-      mask |= 255u << shift;
-      __syncthreads();
-    }
-    t = s_prefix;
-    need = (int)s_k;
+  const int b = blockIdx.x, tid = threadIdx.x;
+  const int64_t lo = p.bt.row_off[b];
+  const int nrows = (int)(p.bt.row_off[b + 1] - lo);
+  const int budget = p.budget[b];
+  if (!p.role) {
+    const int ra = p.bt.reg_off[p.bt.seg_first[b]], rb = p.bt.reg_off[p.bt.seg_first[b + 1]];
+    mark_register_bits(regs, lo, min(nrows, kRegBitRows), p.bt.reg_idx, ra, rb);
   }
-  // contiguous runs of rows per thread keep the tie ranking in row order
-  const int64_t nrows = hi - lo;
-  const int64_t per = (nrows + blockDim.x - 1) / blockDim.x;
-  const int64_t a = lo + min(nrows, (int64_t)tid * per), z = lo + min(nrows, ((int64_t)tid + 1) * per);
-  int ties = 0;
-  for (int64_t r = a; r < z; ++r)
-    if (cand(r) && order_key(p.s[r]) == t) ++ties;
-  int ties_total;
-  int rank = block_exclusive_scan(ties, tmp, &ties_total);
-  for (int64_t r = a; r < z; ++r) {
-    bool k;
-    if (p.role[r] != 0) {
-      k = p.keep_registers != 0;
-    } else if (!cand(r)) {
-      k = false;
-    } else {
-      const uint32_t key = order_key(p.s[r]);
-      if (key == t) {
-        k = rank < need;
-        ++rank;
-      } else {
-        k = key > t;
+  auto is_reg = [&](int i) { return p.role ? p.role[lo + i] != 0 : test_bit(regs, i); };
+  auto global_cand = [&](int i) { return !is_reg(i) && (!p.prev_keep || p.prev_keep[lo + i] != 0); };
+  if (STAGED) {
+    // rows i, i + 1024, ...: a warp's 32 rows are one word of bits. Four
+    // rows' loads in flight per thread.
+    for (int i0 = 0; i0 < nrows; i0 += 4096) {
+      float s[4];
+      bool c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k * 1024 + tid;
+        s[k] = i < nrows ? p.s[lo + i] : 0.f;
+        c[k] = i < nrows && global_cand(i);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k * 1024 + tid;
+        const uint32_t w = __ballot_sync(0xffffffffu, c[k]);
+        if (i < nrows) {
+          keys[i] = order_key(s[k]);
+          if ((tid & 31) == 0) cands[i >> 5] = w;
+        }
       }
     }
-    p.keep[r] = k ? 1 : 0;
+  }
+  auto cand = [&](int i) { return STAGED ? test_bit(cands, i) : global_cand(i); };
+  auto key_of = [&](int i) { return STAGED ? keys[i] : order_key(p.s[lo + i]); };
+  // t = 0 with need = n keeps every candidate (every key is >= 0)
+  uint32_t t = 0, prefix = 0, mask = 0;
+  int need = 0, K = 0;
+  bool select = true;
+  for (int level = 0; level < 3 && select; ++level) {
+    const int shift = level == 0 ? 21 : level == 1 ? 10 : 0;
+    const uint32_t digit = level == 2 ? 1023u : 2047u;
+    hist[tid] = hist[tid + 1024] = 0;
+    __syncthreads();
+    for (int i = tid; i < nrows; i += 1024) {
+      if (!cand(i)) continue;
+      const uint32_t key = key_of(i);
+      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
+    }
+    __syncthreads();
+    // thread t holds buckets 2047 - 2t and 2046 - 2t
+    const int hi = 2047 - 2 * tid;
+    const int chi = (int)hist[hi], clo = (int)hist[hi - 1];
+    int total;
+    const int above = block_exclusive_scan(chi + clo, tmp, &total);
+    int k;
+    if (level == 0) {
+      const int n = total;  // every candidate
+      K = min(max(budget, 0), n);
+      need = n;
+      if (K == 0) {
+        t = 0xffffffffu;
+        need = 0;
+      }
+      select = K > 0 && K < n;
+      if (!select) break;
+      k = K;
+    } else {
+      k = need;
+    }
+    if (above < k && k <= above + chi + clo) {
+      const int bucket = above + chi >= k ? hi : hi - 1;
+      s_k = (uint32_t)(bucket == hi ? k - above : k - above - chi);
+      s_prefix = prefix | ((uint32_t)bucket << shift);
+    }
+    __syncthreads();
+    prefix = s_prefix;
+    need = (int)s_k;
+    mask |= digit << shift;
+    t = prefix;
+  }
+  // whether the keys equal to t are all needed (hist holds the last level's
+  // counts: the bucket of t counts exactly the keys equal to it)
+  __syncthreads();
+  const bool all_ties = !select || (int)hist[t & 1023u] == need;
+  if (all_ties) {
+    for (int i = tid; i < nrows; i += 1024) {
+      bool k = false;
+      if (is_reg(i)) {
+        k = p.keep_registers != 0;
+      } else if (cand(i)) {
+        const uint32_t key = key_of(i);
+        k = key > t || (key == t && need > 0);
+      }
+      p.keep[lo + i] = k ? 1 : 0;
+    }
+  } else {
+    // contiguous runs of rows per thread keep the tie ranking in row order
+    const int per = (nrows + 1023) / 1024;
+    const int a = min(nrows, tid * per), z = min(nrows, a + per);
+    int ties = 0;
+    for (int i = a; i < z; ++i)
+      if (cand(i) && key_of(i) == t) ++ties;
+    int ties_total;
+    int rank = block_exclusive_scan(ties, tmp, &ties_total);
+    for (int i = a; i < z; ++i) {
+      bool k = false;
+      if (is_reg(i)) {
+        k = p.keep_registers != 0;
+      } else if (cand(i)) {
+        const uint32_t key = key_of(i);
+        if (key == t) {
+          k = rank < need;
+          ++rank;
+        } else {
+          k = key > t;
+        }
+      }
+      p.keep[lo + i] = k ? 1 : 0;
+    }
   }
   if (tid == 0 && p.count_vis) p.count_vis[b] = K;
+}
+
+// Samples of up to kBudgetStagedRows rows are staged in shared memory (their
+// keys, 160 KB at most); the bits of larger ones would not fit beside it.
+constexpr int kBudgetStagedRows = 40960;
+static_assert(kBudgetStagedRows <= kRegBitRows, "candidate and register bits");
+
+int launch_budget_keep(const BudgetParams& p, int64_t max_sample_rows, cudaStream_t st) {
+  if (max_sample_rows <= kBudgetStagedRows) {
+    const size_t smem = (size_t)max_sample_rows * 4;
+    if (smem > 16 * 1024 &&
+        cudaFuncSetAttribute(budget_keep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kBudgetStagedRows * 4) != cudaSuccess)
+      return 1;
+    budget_keep_kernel<true><<<p.bt.B, 1024, smem, st>>>(p);
+  } else {
+    budget_keep_kernel<false><<<p.bt.B, 1024, 0, st>>>(p);
+  }
+  count_launch();
+  return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
 // One thread per merged row; the group's values are added in row order.
