@@ -391,9 +391,12 @@ def occam_construct_registers(layout: BatchLayout, h, k_reg, ws=None, stream=Non
     k_reg = _dev_tensor(k_reg, torch.int32, "k_reg")
     if h.dim() != 2 or h.shape[0] != layout.total_rows:
         raise OccamError(OCCAM_ERR_INVALID_ARG, "h must be [total_rows, channels]")
-    if k_reg.numel() and (int(k_reg.min()) < 0 or int(k_reg.max()) >= h.shape[1]):
+    # checked on the host from one copy of the list (min, max and unique on the
+    # device took five kernels and three waits, 110 us of a 197 us call)
+    ks = k_reg.reshape(-1).tolist()
+    if ks and (min(ks) < 0 or max(ks) >= h.shape[1]):
         raise OccamError(OCCAM_ERR_INVALID_ARG, "k_reg channels out of range")
-    if k_reg.numel() != torch.unique(k_reg).numel():
+    if len(set(ks)) != len(ks):
         raise OccamError(OCCAM_ERR_INVALID_ARG, "k_reg channels must be distinct")
     ws = _ws(ws, layout, 1, 1)
     cb = layout.c()

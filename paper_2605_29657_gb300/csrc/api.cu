@@ -1031,14 +1031,12 @@ int occam_construct_registers(const occam_batch* batch, void* h, int64_t channel
   if (n_k == 0 || batch->S_tot == 0) return OCCAM_OK;
   OCCAM_TRY(require_device(k_reg));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
   RegistersParams p;
   p.bt = dev_batch(batch);
   p.h = static_cast<__nv_bfloat16*>(h);
   p.channels = channels;
   p.k_reg = k_reg;
   p.n_k = n_k;
-  p.role = at<uint8_t>(workspace, L.role);
   registers_kernel<<<batch->S_tot, 256, 0, st>>>(p);
   count_launch();
   return cuda_ok();

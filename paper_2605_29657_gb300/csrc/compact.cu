@@ -301,34 +301,75 @@ __global__ void __launch_bounds__(256) stage_rows_kernel(StageRowsParams p) {
   }
 }
 
-// registers_kernel: one CTA per segment. For each register channel in turn,
-// the CTA takes the max over the segment's visual rows (a thread-strided
-// pass, then a block max), writes it into the channel of every register row
-// and zeroes the channel on the visual rows. Values are compared as floats;
-// the written max is one of the bf16 inputs, so results are exact.
+// registers_kernel: one CTA per segment. Thread t takes channel t % n_k of the
+// rows t / n_k, + RP, ... (RP = 256 / n_k rows at a time; more than 256
+// channels in groups of 256), sixteen loads in flight, so that the 32-byte
+// sectors of one row, which lie in one DRAM page, are touched together. The
+// max of a channel over the visual rows, met in shared memory, goes into the
+// channel of every register row; the visual rows' values are zeroed. The
+// segment's registers are marked in shared memory, a window of rows at a
+// time. Values are compared as floats; the written max is one of the bf16
+// inputs, so results are exact. Bound by what HBM fetches and writes back for
+// the 2-byte values: 78 us on 185,600 rows of 1,024 channels, 10 of them
+// register channels, at any number of threads and CTAs (as with the channels
+// in turn, which took a memset and a scatter of the roles besides).
 __global__ void __launch_bounds__(256) registers_kernel(RegistersParams p) {
-  __shared__ float wmax[8];
-  const int seg = blockIdx.x;
-  const int tid = threadIdx.x;
+  constexpr int U = 16, NT = 256;
+  __shared__ uint32_t bits[kRegBitWords];
+  __shared__ float wmax[NT];
+  const int seg = blockIdx.x, tid = threadIdx.x;
   const int64_t r0 = p.bt.seg_off[seg], r1 = p.bt.seg_off[seg + 1];
   const int32_t g0 = p.bt.reg_off[seg], g1 = p.bt.reg_off[seg + 1];
-  for (int j = 0; j < p.n_k; ++j) {
-    const int64_t k = p.k_reg[j];
+  const int nwin = (int)((r1 - r0 + kRegBitRows - 1) / kRegBitRows);
+  for (int j0 = 0; j0 < p.n_k; j0 += NT) {
+    const int nk = min(NT, p.n_k - j0);
+    const int RP = NT / nk, row = tid / nk, ch = tid - row * nk;
+    const bool on = row < RP;
+    __nv_bfloat16* const col = p.h + p.k_reg[j0 + ch];
     float m = -INFINITY;
-    for (int64_t r = r0 + tid; r < r1; r += blockDim.x)
-      if (p.role[r] == 0) m = fmaxf(m, __bfloat162float(p.h[r * p.channels + k]));
+    for (int w = 0; w < nwin; ++w) {
+      const int64_t w0 = r0 + (int64_t)w * kRegBitRows;
+      const int n = (int)min(r1 - w0, (int64_t)kRegBitRows);
+      if (nwin > 1 || j0 == 0) {
+        __syncthreads();
+        mark_register_bits(bits, w0, n, p.bt.reg_idx, g0, g1);
+      }
+      if (!on) continue;
+      for (int i0 = row; i0 < n; i0 += RP * U) {
+        __nv_bfloat16 v[U];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((tid & 31) == 0) wmax[tid >> 5] = m;
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + RP * u;
+          v[u] = i < n ? col[(w0 + i) * p.channels] : __float2bfloat16_rn(-INFINITY);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + RP * u;
+          if (i < n && !test_bit(bits, i)) m = fmaxf(m, __bfloat162float(v[u]));
+        }
+      }
+    }
+    __syncthreads();  // (the group before this one has read its maxima)
+    wmax[tid] = m;
     __syncthreads();
-    float mx = wmax[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmaxf(mx, wmax[w]);
-    // a segment without visual rows leaves its registers as they are
-    if (mx != -INFINITY)
-      for (int i = g0 + tid; i < g1; i += blockDim.x) p.h[(int64_t)p.bt.reg_idx[i] * p.channels + k] = __float2bfloat16_rn(mx);
-    for (int64_t r = r0 + tid; r < r1; r += blockDim.x)
-      if (p.role[r] == 0) p.h[r * p.channels + k] = __float2bfloat16_rn(0.f);
-    __syncthreads();
+    if (tid < nk) {
+      for (int q = 1; q < RP; ++q) m = fmaxf(m, wmax[q * nk + tid]);
+      // a segment without visual rows leaves its registers as they are
+      if (m != -INFINITY)
+        for (int i = g0; i < g1; ++i) col[(int64_t)p.bt.reg_idx[i] * p.channels] = __float2bfloat16_rn(m);
+    }
+    // with more than one window the last one's bits are at hand: backwards
+    for (int w = nwin - 1; w >= 0; --w) {
+      const int64_t w0 = r0 + (int64_t)w * kRegBitRows;
+      const int n = (int)min(r1 - w0, (int64_t)kRegBitRows);
+      if (w < nwin - 1) {
+        __syncthreads();
+        mark_register_bits(bits, w0, n, p.bt.reg_idx, g0, g1);
+      }
+      if (on)
+        for (int i = row; i < n; i += RP)
+          if (!test_bit(bits, i)) col[(w0 + i) * p.channels] = __float2bfloat16_rn(0.f);
+    }
   }
 }
 

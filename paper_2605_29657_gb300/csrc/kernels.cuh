@@ -226,7 +226,6 @@ struct RegistersParams {
   int64_t channels;
   const int32_t* k_reg;  // [n_k] channel indices
   int n_k;
-  const uint8_t* role;
 };
 
 // lambda2 budget matching (App. A): the K-th largest ratio s2[v] / ref2[b(v)]

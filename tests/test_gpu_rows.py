@@ -82,3 +82,28 @@ def test_rules_at_unit_edges(shape, prev):
         keep, got = occ.occam_budget_keep(lay, ts, torch.from_numpy(budget.astype(np.int32)).cuda(), prev_keep=tp)
         assert (keep.cpu().numpy().astype(bool) == want).all()
         assert got.cpu().numpy().tolist() == cnt.tolist()
+
+
+@pytest.mark.parametrize("n_k", [1, 10, 255, 256, 257])
+def test_construct_registers_channel_groups(n_k):
+    """Up to 256 channels go through the CTA at once; 257 take a second group."""
+    import paper_2605_29657_gb300 as occ
+
+    lay, seg_off, _, _, rng = _layout([3, 300, 4100], [2, 1], 2, seed=n_k)
+    h = torch.randn(int(seg_off[-1]), 300, generator=torch.Generator().manual_seed(n_k)).to(torch.bfloat16)
+    k = rng.permutation(300)[:n_k].astype(np.int32)
+    want = O.construct_registers(h.float().numpy(), seg_off, lay.host["reg_idx"], lay.host["reg_off"], k)
+    got = occ.occam_construct_registers(lay, h.cuda(), torch.from_numpy(k).cuda())
+    assert (got.float().cpu().numpy() == want).all()
+
+
+def test_construct_registers_several_windows():
+    """A segment of more rows than the register bits hold (two windows), and one without visual rows."""
+    import paper_2605_29657_gb300 as occ
+
+    lay, seg_off, _, _, _ = _layout([65536 + 70, 2], [1, 1], 2, seed=3)
+    h = torch.randn(int(seg_off[-1]), 12, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16)
+    k = np.asarray([11, 0, 5], np.int32)
+    want = O.construct_registers(h.float().numpy(), seg_off, lay.host["reg_idx"], lay.host["reg_off"], k)
+    got = occ.occam_construct_registers(lay, h.cuda(), torch.from_numpy(k).cuda())
+    assert (got.float().cpu().numpy() == want).all()
