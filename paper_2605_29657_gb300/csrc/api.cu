@@ -1053,7 +1053,6 @@ int occam_calibrate_lambda2(const occam_batch* batch, const float* s2, const flo
   WsLayout L;
   OCCAM_TRY(check_ws(batch, 1, 1, workspace, workspace_bytes, &L));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
   Lambda2Params p;
   p.bt = dev_batch(batch);
   p.s2 = s2;
@@ -1065,6 +1064,11 @@ int occam_calibrate_lambda2(const occam_batch* batch, const float* s2, const flo
   p.sel = at<unsigned char>(workspace, L.l2sel);
   p.lambda2 = lambda2_out;
   p.n_candidates = n_candidates;
+  if (batch->total_rows <= kL2ClusterRows) {
+    if (launch_l2_cluster(p, st) != 0) return OCCAM_ERR_CUDA;
+    return cuda_ok();
+  }
+  OCCAM_TRY(mark_roles(batch, L, workspace, st));
   // keys and top-digit histogram, then per digit a one-CTA bucket choice and
   // the next digit's histogram, the window of kept counts, the choice
   OCCAM_CUDA(cudaMemsetAsync(p.sel, 0, kL2SelBytes, st));

@@ -13,8 +13,10 @@
 //   offsets are staged in shared memory for the per-row sample lookups.
 // gather_kernel: persistent grid; one warp copies one kept row of one tensor
 //   with 16-byte loads / stores (exact bit copy).
+#include <cooperative_groups.h>
 #include <cuda.h>
 
+#include <cuda/std/type_traits>
 #include <mutex>
 
 #include "common.cuh"
@@ -427,11 +429,13 @@ __device__ __forceinline__ uint32_t l2_mask_above(int level) {
   return level == 0 ? 0u : level == 1 ? 0xFFE00000u : 0xFFFFFC00u;
 }
 
-// lambda0 stepped by j fp32 steps (j < 0: down, toward 0)
+// lambda0 (>= 0) stepped by j fp32 steps (j < 0: down, toward 0), as |j| calls
+// of nextafterf would, by its bit pattern (the calls' instructions were 25 of
+// the 28 us of the window's pass)
 __device__ __forceinline__ float l2_step(float lam, int j) {
-  for (; j < 0; ++j) lam = nextafterf(lam, 0.f);
-  for (; j > 0; --j) lam = nextafterf(lam, __int_as_float(0x7f800000));
-  return lam;
+  const int bits = __float_as_int(lam);
+  if (bits > 0x7f800000) return lam;  // no number
+  return __int_as_float(min(max(bits + j, 0), 0x7f800000));
 }
 }  // namespace
 
@@ -584,6 +588,282 @@ __global__ void __launch_bounds__(1024) l2_finish_kernel(Lambda2Params p) {
   }
   __syncthreads();
   if (threadIdx.x == 0) *p.lambda2 = s_lam;
+}
+
+// The same selection by one cluster of 16 CTAs, for up to kL2ClusterRows rows:
+// CTA r takes the r-th sixteenth of the rows and keeps their keys in shared
+// memory, so each digit costs a pass over shared memory, the sums of the
+// buckets over the cluster (distributed shared memory), the choice in CTA 0
+// and three cluster barriers. Bound by that chain; the grid-wide
+// kernels above pay a launch per step (74 us a call on 185,600 rows).
+namespace {
+constexpr int kL2Threads = 1024;
+constexpr int kL2Staged = 512;  // samples whose offsets and references are kept in shared memory
+struct L2Shared {
+  uint32_t hist[3][kL2Digits];
+  uint32_t tot[kL2Digits];  // CTA 0: the level's buckets over the cluster
+  uint32_t part[kL2Threads];
+  uint32_t regs[kL2ClusterRows / kL2ClusterCtas / 32];
+  int64_t ro[kL2Staged + 1];
+  float ref[kL2Staged];
+  unsigned long long kept[2 * kL2Window + 1];
+  int n, cnt;
+  float min_ref;  // CTA 0: the smallest positive reference
+  // written by CTA 0 into every CTA
+  uint32_t prefix;
+  int k, done;
+  int tmp[40];
+};
+}  // namespace
+
+__global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p) {
+  extern __shared__ uint32_t l2_keys[];
+  __shared__ L2Shared sm;
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
+  L2Shared* const root = cluster.map_shared_rank(&sm, 0);
+  const int64_t R = p.bt.total_rows;
+  const int64_t chunk = (R + kL2ClusterCtas - 1) / kL2ClusterCtas;
+  const int64_t c0 = min(R, rank * chunk), c1 = min(R, c0 + chunk);
+  const int n = (int)(c1 - c0);
+  const bool staged = p.bt.B <= kL2Staged;
+  constexpr int NW = 2 * kL2Window + 1;
+  for (int i = tid; i < 3 * kL2Digits; i += kL2Threads) (&sm.hist[0][0])[i] = 0;
+  for (int i = tid; i < (n + 31) / 32; i += kL2Threads) sm.regs[i] = 0;
+  if (staged) {
+    for (int b = tid; b <= p.bt.B; b += kL2Threads) sm.ro[b] = p.bt.row_off[b];
+    if (tid < p.bt.B) sm.ref[tid] = p.ref2[tid];
+  }
+  if (rank == 0 && tid < 32) {
+    float m = INFINITY;
+    for (int b = tid; b < p.bt.B; b += 32) {
+      const float r = p.ref2[b];
+      if (r > 0.f) m = fminf(m, r);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (tid == 0) sm.min_ref = m;
+  }
+  if (tid < NW) sm.kept[tid] = 0;
+  if (tid == 0) {
+    sm.n = sm.cnt = 0;
+    sm.done = 0;
+  }
+  __syncthreads();
+  // the registers among this CTA's rows
+  for (int s = tid; s < p.bt.S_tot; s += kL2Threads) {
+    if (p.bt.seg_off[s] < c1 && p.bt.seg_off[s + 1] > c0) {
+      for (int i = p.bt.reg_off[s]; i < p.bt.reg_off[s + 1]; ++i) {
+        const int64_t r = p.bt.reg_idx[i] - c0;
+        if (r >= 0 && r < n) atomicOr(&sm.regs[r >> 5], 1u << (r & 31));
+      }
+    }
+  }
+  // CTA 0's counters are zeroed before anything is added to them
+  cluster.sync();
+  const int64_t* ro = staged ? sm.ro : p.bt.row_off;
+  const float* ref2 = staged ? sm.ref : p.ref2;
+  // keys, and the histogram of their top digit; eight rows' loads and sample
+  // searches at once per thread
+  int cand = 0;
+  int steps = 0;
+  while ((1 << steps) < p.bt.B) ++steps;
+  for (int i0 = tid; i0 < n; i0 += 8 * kL2Threads) {
+    float s[8];
+    bool c[8];
+    int lo[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * kL2Threads;
+      s[u] = i < n ? p.s2[c0 + i] : 0.f;
+      c[u] = i < n && p.keep1[c0 + i] != 0;
+      lo[u] = 0;
+    }
+    // the largest b with ro[b] <= row
+    for (int h = steps - 1; h >= 0; --h) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int b = lo[u] + (1 << h);
+        if (b < p.bt.B && ro[b] <= c0 + i0 + u * kL2Threads) lo[u] = b;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * kL2Threads;
+      uint32_t key = 0;
+      if (c[u] && !test_bit(sm.regs, i)) {
+        const float ref = ref2[lo[u]];
+        if (ref > 0.f) {
+          key = 0x80000000u | __float_as_uint(__fdiv_rn(s[u], ref));
+          ++cand;
+          atomicAdd(&sm.hist[0][key >> 21], 1u);
+        }
+      }
+      if (i < n) l2_keys[i] = key;
+    }
+  }
+  cand = __reduce_add_sync(0xffffffffu, cand);
+  if ((tid & 31) == 0 && cand) atomicAdd(&root->n, cand);
+  for (int level = 0; level < 3; ++level) {
+    if (level > 0) {
+      const uint32_t prefix = sm.prefix, mask = l2_mask_above(level);
+      const int shift = l2_shift(level);
+      for (int i = tid; i < n; i += kL2Threads) {
+        const uint32_t key = l2_keys[i];
+        if ((key >> 31) && (key & mask) == prefix) atomicAdd(&sm.hist[level][(key >> shift) & (kL2Digits - 1)], 1u);
+      }
+    }
+    cluster.sync();
+    {
+      // CTA r adds up the r-th sixteenth of the buckets over the cluster
+      // (each thread one bucket of two CTAs) and gives the sums to CTA 0
+      constexpr int SL = kL2Digits / kL2ClusterCtas;
+      static_assert(SL * kL2ClusterCtas / 2 == kL2Threads, "two CTAs' buckets per thread");
+      const int b = rank * SL + tid % SL, q = tid / SL * 2;
+      sm.part[tid] = cluster.map_shared_rank(&sm, q)->hist[level][b] + cluster.map_shared_rank(&sm, q + 1)->hist[level][b];
+      __syncthreads();
+      if (tid < SL) {
+        uint32_t t = 0;
+#pragma unroll
+        for (int u = 0; u < kL2ClusterCtas / 2; ++u) t += sm.part[u * SL + tid];
+        root->tot[b] = t;
+      }
+    }
+    cluster.sync();
+    if (rank == 0) {
+      bool go = true;
+      if (level == 0) {
+        const int total = sm.n;
+        if (tid == 0 && p.n_candidates) *p.n_candidates = total;
+        if (p.target <= 0 || p.target > total) {
+          // K <= 0: no lambda2 keeps nothing but +inf; K > n: 0 keeps every candidate
+          go = false;
+          if (tid == 0) *p.lambda2 = p.target <= 0 ? __int_as_float(0x7f800000) : 0.f;
+          if (tid < kL2ClusterCtas) cluster.map_shared_rank(&sm, tid)->done = 1;
+        }
+      }
+      if (go) {
+        // thread t holds buckets 2047 - 2t and 2046 - 2t
+        const int k = level == 0 ? (int)p.target : sm.k;
+        const uint32_t prefix = level == 0 ? 0u : sm.prefix;
+        const int hi = kL2Digits - 1 - 2 * tid;
+        const int chi = (int)sm.tot[hi], clo = (int)sm.tot[hi - 1];
+        int total;
+        const int above = block_exclusive_scan(chi + clo, sm.tmp, &total);
+        if (above < k && k <= above + chi + clo) {
+          const int bucket = above + chi >= k ? hi : hi - 1;
+          const uint32_t pf = prefix | ((uint32_t)bucket << l2_shift(level));
+          const int kr = bucket == hi ? k - above : k - above - chi;
+          for (int r = 0; r < kL2ClusterCtas; ++r) {
+            L2Shared* const q = cluster.map_shared_rank(&sm, r);
+            q->prefix = pf;
+            q->k = kr;
+          }
+        }
+      }
+    }
+    cluster.sync();
+    if (sm.done) return;  // (every CTA alike; nothing remote is in flight)
+  }
+  // Kept counts of the selected ratio and its neighbours. A row whose
+  // quotient lies more than 128 fp32 steps off every lambda tested (2^-17 of
+  // it and more) passes or fails the product test by a margin far above the
+  // roundings of quotient and product (2^-24 each, as long as neither is
+  // subnormal): only nearer rows are evaluated.
+  const float lam0 = __uint_as_float(sm.prefix & 0x7fffffffu);
+  const bool margin = lam0 > 1e-30f && lam0 * root->min_ref > 1e-30f;
+  auto kept_at = [&](const float* lam, int* c, auto count) {
+    const float first = lam[0], last = lam[decltype(count)::value - 1];
+    for (int i = tid; i < n; i += kL2Threads) {
+      const uint32_t key = l2_keys[i];
+      if (key >> 31) {
+        const int q = (int)(key & 0x7fffffffu);
+        if (margin && q < __float_as_int(first) - 128) continue;
+        if (margin && q > __float_as_int(last) + 128) {
+#pragma unroll
+          for (int j = 0; j < decltype(count)::value; ++j) ++c[j];
+          continue;
+        }
+        const int64_t r = c0 + i;
+        const float s = p.s2[r], ref = ref2[upper_interval(ro, p.bt.B, r)];
+#pragma unroll
+        for (int j = 0; j < decltype(count)::value; ++j) c[j] += s >= __fmul_rn(lam[j], ref) ? 1 : 0;
+      }
+    }
+  };
+  {
+    float lam[NW];
+    int c[NW];
+#pragma unroll
+    for (int j = 0; j < NW; ++j) {
+      lam[j] = l2_step(lam0, j - kL2Window);
+      c[j] = 0;
+    }
+    kept_at(lam, c, cuda::std::integral_constant<int, NW>());
+#pragma unroll
+    for (int j = 0; j < NW; ++j) {
+      const int v = __reduce_add_sync(0xffffffffu, c[j]);
+      if ((tid & 31) == 0 && v) atomicAdd(&sm.kept[j], (unsigned long long)v);
+    }
+    __syncthreads();
+    if (rank != 0 && tid < NW && sm.kept[tid]) atomicAdd(&root->kept[tid], sm.kept[tid]);
+  }
+  cluster.sync();
+  const int64_t K = p.target;
+  // every CTA follows the same steps from CTA 0's counts
+  unsigned long long kept[NW];
+#pragma unroll
+  for (int j = 0; j < NW; ++j) kept[j] = root->kept[j];
+  float lam = 0.f;
+  const bool below = (int64_t)kept[0] < K, above = !below && (int64_t)kept[NW - 1] >= K;
+  if (!below && !above) {
+    int j = NW - 1;
+    while ((int64_t)kept[j] < K) --j;  // kept is non-increasing in lambda2; kept[0] >= K
+    lam = l2_step(lam0, j - kL2Window);
+  } else {
+    // beyond the window: single steps down while fewer than K are kept
+    // (kept(0) counts every candidate), or up while the next value keeps K
+    lam = l2_step(lam0, below ? -kL2Window : kL2Window);
+    for (int it = 0; it < 64; ++it) {
+      const float next = l2_step(lam, below ? -1 : 1);
+      if (rank == 0 && tid == 0) sm.cnt = 0;
+      cluster.sync();
+      int c = 0;
+      kept_at(&next, &c, cuda::std::integral_constant<int, 1>());
+      c = __reduce_add_sync(0xffffffffu, c);
+      if ((tid & 31) == 0 && c) atomicAdd(&root->cnt, c);
+      cluster.sync();
+      const bool keeps = root->cnt >= K;
+      if (below || keeps) lam = next;
+      if (below == keeps) break;  // (no CTA resets cnt before every CTA has read it: the sync below)
+      cluster.sync();
+    }
+  }
+  if (rank == 0 && tid == 0) *p.lambda2 = lam;
+  cluster.sync();  // CTA 0's counts are read until here
+}
+
+int launch_l2_cluster(const Lambda2Params& p, cudaStream_t st) {
+  const int64_t chunk = (p.bt.total_rows + kL2ClusterCtas - 1) / kL2ClusterCtas;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kL2ClusterCtas);
+  cfg.blockDim = dim3(kL2Threads);
+  cfg.dynamicSmemBytes = (size_t)chunk * 4;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kL2ClusterCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(l2_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(l2_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kL2ClusterRows / kL2ClusterCtas * 4)) != cudaSuccess)
+    return 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, l2_cluster_kernel, p) == cudaSuccess ? 0 : 1;
 }
 
 }  // namespace occam

@@ -244,6 +244,10 @@ struct Lambda2Params {
 };
 constexpr int kL2Digits = 2048;         // lambda2 selection: 11-bit digits
 constexpr int kL2Window = 4;            // fp32 steps either way whose kept counts are taken in one pass
+// up to this many rows lambda2 is selected by one cluster of 16 CTAs that
+// keeps every row's key in shared memory; above, by grid-wide passes
+constexpr int kL2ClusterCtas = 16;
+constexpr int64_t kL2ClusterRows = (int64_t)kL2ClusterCtas * 40960;
 constexpr int kL2SelBytes = 32 * 1024;  // workspace scratch of the selection
 
 // mean-threshold reference (component ablation): ref[u] = mean of s over the
@@ -333,6 +337,7 @@ __global__ void l2_select_kernel(Lambda2Params p, int level);
 __global__ void l2_window_kernel(Lambda2Params p);
 __global__ void l2_finish_kernel(Lambda2Params p);
 __global__ void registers_kernel(RegistersParams p);
+int launch_l2_cluster(const Lambda2Params& p, cudaStream_t st);
 
 // rules.cu
 __global__ void mean_ref_kernel(MeanRefParams p);

@@ -107,3 +107,33 @@ def test_construct_registers_several_windows():
     want = O.construct_registers(h.float().numpy(), seg_off, lay.host["reg_idx"], lay.host["reg_off"], k)
     got = occ.occam_construct_registers(lay, h.cuda(), torch.from_numpy(k).cuda())
     assert (got.float().cpu().numpy() == want).all()
+
+
+@pytest.mark.parametrize("seg_rows,segs", [
+    ([5], [1]),                                  # fewer rows than CTAs
+    ([17, 1, 300], [1, 2]),
+    ([3] * 1200, [2] * 600),                     # more samples than are staged
+    ([100000, 227680], [1, 1]),
+    ([655360], [1]),                             # the most rows of the one-cluster kernel
+    ([655361], [1]),                             # the grid-wide kernels
+])
+def test_calibrate_lambda2_row_ranges(seg_rows, segs):
+    import paper_2605_29657_gb300 as occ
+
+    lay, _, row_off, is_reg, rng = _layout(seg_rows, segs, 1, seed=len(seg_rows))
+    n, B = int(row_off[-1]), len(segs)
+    for spread, tiny in ((1.0, False), (1e-4, False), (1.0, True)):
+        # wide, nearly tied (many quotients within the window), and products too small for the margin shortcut
+        s2 = np.exp(spread * rng.standard_normal(n)).astype(np.float32)
+        ref2 = np.exp(0.2 * rng.standard_normal(B)).astype(np.float32)
+        if tiny:
+            s2, ref2 = s2 * np.float32(1e-33), ref2 * np.float32(1e-16)
+        ref2[rng.random(B) < 0.1] = 0
+        keep1 = (rng.random(n) < 0.4).astype(np.uint8)
+        args = [torch.from_numpy(x).cuda() for x in (s2, ref2, keep1)]
+        nc = int((keep1.astype(bool) & ~is_reg & (ref2[np.repeat(np.arange(B), np.diff(row_off))] > 0)).sum())
+        for K in sorted({0, 1, nc // 7, nc - 1, nc, nc + 1}):
+            want, cnt = O.lambda2_for_budget(s2, ref2, keep1, is_reg, row_off, K)
+            lam, got = occ.occam_calibrate_lambda2(lay, *args, K)
+            assert int(got[0]) == cnt == nc
+            assert np.float32(lam[0].item()) == want, (K, spread, tiny)
