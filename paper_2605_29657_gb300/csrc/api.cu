@@ -386,11 +386,20 @@ int launch_stage1_scores(const occam_batch* b, const occam_stage1_args* a, const
         !encode_map3(&mq1, a->q, b->total_rows, a->H1, a->d1, 16) ||
         !encode_map3(&mk1, a->K1, b->total_rows, a->H1, a->d1, 16))
       return OCCAM_ERR_CUDA;
-    p.tiles = (int)cdiv(b->max_seg_rows, 128);
-    p.hgroups = (int)cdiv(a->H1, kMutHeadGroup);
+    p.tiles = (int)cdiv(b->max_seg_rows, kMutTileRows);
+    // heads per item of the second pass: 4 (fewer item ends), less where the
+    // batch would give a CTA pair under 12 items (at 6 images of 353-1,709
+    // rows, 12 heads: 96 items of 4 heads for 76 pairs, whose longest pair
+    // gets 1.6 times the mean; 1.08 with one head each)
+    const int64_t mut_tiles = cdiv(b->total_rows, kMutTileRows) + b->S_tot / 2;
+    p.hgsize = 4;
+    while (p.hgsize > 1 && mut_tiles * cdiv(a->H1, p.hgsize) < 6 * (int64_t)num_sms()) p.hgsize >>= 1;
+    p.hgroups = (int)cdiv(a->H1, p.hgsize);
     p.part = p.lsum + (int64_t)a->H1 * b->total_rows;  // stats1 holds 2 * H1 floats per row
     p.queue = at<int32_t>(ws, L.counters) + CNT_MUT;
-    OCCAM_CUDA(cudaMemsetAsync(p.queue, 0, 2 * sizeof(int32_t), st));
+    p.n_redo = p.queue + 3;
+    p.redo = reinterpret_cast<int32_t*>(p.part);
+    OCCAM_CUDA(cudaMemsetAsync(p.queue, 0, 4 * sizeof(int32_t), st));
     launch_mutual_tc(p, mq, mk, mq1, mk1, num_sms(), st);
     trace.mark(st);
   }

@@ -270,9 +270,9 @@ enum {
   CNT_SEG_TICKET = 8,  // Stage-I finalize: segment order
   CNT_NF16 = 9,
   CNT_QUEUE16 = 10,    // next fused Stage-II item (16-CTA clusters)
-  CNT_MUT = 11,        // [2] next mutual Stage-I item of each pass
-  CNT_NHS = 13,        // Stage-II text tiles split over head groups (merge items)
-  CNT_SLOTS = 14
+  CNT_MUT = 11,        // [3] next mutual Stage-I item of each pass and of the redo of pass 1; [1] items to redo
+  CNT_NHS = 15,        // Stage-II text tiles split over head groups (merge items)
+  CNT_SLOTS = 16
 };
 
 constexpr int kTextTile = 64;    // Stage-II text rows per item of the two-pass score pass

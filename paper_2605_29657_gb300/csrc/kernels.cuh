@@ -69,12 +69,15 @@ struct MutualTcParams {
   float* s1;
   float* s2_zero;    // nullable
   int* status;
-  int tiles;         // 128-row tiles of the longest segment
-  int32_t* queue;    // [2] work-queue heads of the two passes, zero before the launch
-  int hgroups;       // head groups of kMutHeadGroup heads (second pass)
+  int tiles;         // tiles of kMutTileRows rows of the longest segment
+  int32_t* queue;    // [3] work-queue heads of the two passes and of pass 1's redo, zero before the launch
+  int32_t* n_redo;   // pass-1 items to redo: their count (zero before the launch) ...
+  int32_t* redo;     // ... and numbers (at most one per head and 32 rows of a segment; in part's place)
+  int hgsize;        // heads per work item of the second pass
+  int hgroups;       // ... and groups of that many heads
   float* part;       // [hgroups, total_rows] each head group's share of s1
 };
-constexpr int kMutHeadGroup = 4;
+constexpr int kMutTileRows = 256;  // rows of a work item (a pair of CTAs, 128 each)
 
 
 struct ThresholdParams {

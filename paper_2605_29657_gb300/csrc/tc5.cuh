@@ -39,6 +39,18 @@ __device__ __forceinline__ void bar_arrive_remote(uint64_t* b, uint32_t rank) {
       "r"(rank)
       : "memory");
 }
+// the same without the cluster-scope release, whose fence costs the arriving
+// warp hundreds of cycles: for arrivals that publish no generic-proxy data
+// (tiles that TMA or fence.proxy.async already ordered, TMEM reads that
+// tcgen05.fence orders)
+__device__ __forceinline__ void bar_signal_remote(uint64_t* b, uint32_t rank) {
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\t"
+      "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
+      "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(su32(b)),
+      "r"(rank)
+      : "memory");
+}
 __device__ __forceinline__ bool bar_try(uint64_t* b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -62,16 +74,24 @@ __device__ __forceinline__ bool bar_try_cluster(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: gives up after `limit_ns` of wall time or as soon as *abort
-// becomes non-zero. Returns true when the phase completed.
+// Bounded wait: gives up after `limit_ns` of wall time (counted from its 64th
+// unsuccessful try: the timer is slow to read, and nearly every wait ends
+// before) or as soon as *abort becomes non-zero. Returns true when the phase
+// completed.
 __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, volatile int* abort, uint64_t limit_ns,
                                          bool cluster_scope = false) {
   if (cluster_scope ? bar_try_cluster(b, parity) : bar_try(b, parity)) return true;
-  const uint64_t t0 = globaltimer();
+  uint64_t t0 = 0;
   for (uint32_t it = 1;; ++it) {
     if (cluster_scope ? bar_try_cluster(b, parity) : bar_try(b, parity)) return true;
     if (abort && *abort) return false;
-    if ((it & 255u) == 0 && globaltimer() - t0 > limit_ns) return false;
+    if ((it & 63u) == 0) {
+      const uint64_t t = globaltimer();
+      if (t0 == 0)
+        t0 = t;
+      else if (t - t0 > limit_ns)
+        return false;
+    }
   }
 }
 
@@ -151,6 +171,35 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accum)
       : "memory");
+}
+// The CTA-pair forms (cta_group::2): one thread of the pair's leader (the CTA
+// of even rank) issues an MMA over both CTAs' tensor cores. A and B each lie
+// half in either CTA's shared memory at the same offsets (A: 128 of the 256
+// rows, B: N / 2 of the N rows), and each CTA's TMEM receives its 128 rows.
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accum)
+      : "memory");
+}
+// arrives on the barrier at this offset in both CTAs of a 2-CTA cluster once
+// every MMA issued so far by this thread has completed
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(su32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+// both CTAs of the pair execute these, one warp each
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* holder, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(holder)), "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
