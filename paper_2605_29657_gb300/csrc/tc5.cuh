@@ -74,24 +74,18 @@ __device__ __forceinline__ bool bar_try_cluster(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: gives up after `limit_ns` of wall time (counted from its 64th
-// unsuccessful try: the timer is slow to read, and nearly every wait ends
-// before) or as soon as *abort becomes non-zero. Returns true when the phase
-// completed.
+// Bounded wait: gives up after `limit_ns` of wall time or as soon as *abort
+// becomes non-zero. Returns true when the phase completed. (Reading the timer
+// at the first unsuccessful try also spaces out the polling: read only from
+// the 64th try on, the fused Stage II of 8 and 64 samples took 1-2 % longer.)
 __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, volatile int* abort, uint64_t limit_ns,
                                          bool cluster_scope = false) {
   if (cluster_scope ? bar_try_cluster(b, parity) : bar_try(b, parity)) return true;
-  uint64_t t0 = 0;
+  const uint64_t t0 = globaltimer();
   for (uint32_t it = 1;; ++it) {
     if (cluster_scope ? bar_try_cluster(b, parity) : bar_try(b, parity)) return true;
     if (abort && *abort) return false;
-    if ((it & 63u) == 0) {
-      const uint64_t t = globaltimer();
-      if (t0 == 0)
-        t0 = t;
-      else if (t - t0 > limit_ns)
-        return false;
-    }
+    if ((it & 255u) == 0 && globaltimer() - t0 > limit_ns) return false;
   }
 }
 
