@@ -63,17 +63,16 @@ WsLayout ws_layout(const occam_batch* b, int H1, int H2) {
   const int64_t chmax = cdiv(b->max_sample_rows, kKeyChunk);
   L.maxA = B * tps * nhg * kStatSplits;
   L.maxB = B * tps * chmax;
-  // fused items: one per text tile, or kHsGroups per tile of a head-split batch
-  L.maxF = std::max<int64_t>(B * cdiv(b->max_text, 128), kHsMaxTiles * kHsGroups);
+  // fused items: one per text tile, or several per tile of a head-split batch (each CTA of theirs has a slot)
+  L.maxF = std::max<int64_t>(B * cdiv(b->max_text, 128), kHsSlots);
   L.maxSlots = L.maxB + L.maxF * kFusedSlotsPerItem16;
   L.itemsF = take(L.maxF * 16);
   L.itemsF8 = take(L.maxF * 16);
   L.itemsF16 = take(L.maxF * 16);
   L.itemsHS = take(kHsMaxTiles * 16);
-  // head-split scratch only for batches with at most kHsMaxTiles text tiles
-  L.ppart = (B * cdiv(b->max_text, kHsRows) <= kHsMaxTiles)
-                ? take((size_t)kHsMaxTiles * kHsGroups * 16 * kHsRows * kFusedMaxOwnImg * 4)
-                : 0;
+  // head-split scratch only for batches that can have as few as kHsMaxTiles
+  // text tiles (each sample has one at least)
+  L.ppart = B <= kHsMaxTiles ? take((size_t)kHsSlots * kHsRows * kFusedMaxOwnImg * 4) : 0;
   L.itemA_off = take((B + 1) * 4);
   L.itemB_off = take((B + 1) * 4);
   L.slot_off = take((B + 1) * 4);
@@ -517,10 +516,15 @@ Stage2Params stage2_params(const occam_batch* b, const occam_stage2_args* a, con
   p.slot_off = at<int32_t>(ws, L.slot_off);
   p.maxF = L.maxF;
   p.use_fused = fused ? 1 : 0;
-  p.res16 = widening_enabled() ? fused_resident_clusters(16) : 0;
+  p.res16 = widening_enabled() ? std::min(fused_resident_clusters(16), kHsSlots / 16) : 0;
   p.itemsHS = at<int4>(ws, L.itemsHS);
   p.has_ppart = L.ppart != 0 ? 1 : 0;
   p.res8 = widening_enabled() ? fused_resident_clusters(8) : 0;
+  p.hs_valid = 0;
+  for (int g = 2; g <= kHsGroups; ++g)
+    if (a->H2 % g == 0 && a->H2 / g >= 4 && (a->H2 / g) % (a->H2 / p.Hkv) == 0) p.hs_valid |= 1u << g;
+  // (a split's CTAs need a slot each)
+  p.res4 = widening_enabled() ? std::min(fused_resident_clusters(kFusedCluster), kHsSlots / kFusedCluster) : 0;
   return p;
 }
 
@@ -539,7 +543,7 @@ int fused_launch_clusters(int C, int64_t max_items, int sms) {
 }
 
 int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayout& L, void* ws, float* s2,
-                  float* ref2, float lambda2, cudaStream_t st, Trace trace = Trace()) {
+                  float* ref2, float lambda2, cudaStream_t st, Trace trace = Trace(), bool pdl = false) {
   const NvtxRange nvtx("stage2_scores");
   const Stage2Params p = stage2_params(b, a, L, ws, s2, ref2, lambda2);
   const bool fused = p.use_fused != 0;
@@ -580,24 +584,40 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     q.tau2 = p.tau2;
     q.lambda2 = lambda2;
     q.status = p.status;
+    // A batch whose every text tile fits as a resident 16-CTA cluster takes
+    // 16-CTA clusters for all of its fused samples (the plan's widening; a
+    // sample that a 16-CTA cluster cannot hold fits no smaller one) or, with
+    // more than one tile, 4-CTA clusters with split heads: a launch that can
+    // have no items is not made.
+    const int64_t max_tiles = (int64_t)b->B * cdiv(b->max_text, 128);
+    const bool no8 = p.res16 > 0 && max_tiles <= p.res16;
+    const bool no4 = no8 && (max_tiles == 1 || !q.ppart);
+    // Samples that a 16-CTA cluster holds with all their rows in S1 take no
+    // two-pass kernels.
+    const bool no2p = fused_fits(16, b->max_sample_rows, b->max_text, a->H2);
+    // With the 16-CTA launch alone (one text tile) nothing runs beside it: no
+    // second stream, and it follows the finalize kernel with programmatic
+    // dependent launch.
+    const bool alone = no4 && no2p;
+    q.pdl = 0;
     // The 8-CTA launch runs beside the 4-CTA one on a second stream (fork and
     // join by events), so SMs one of them leaves idle serve the other. Both
     // launch a cluster per SM group; clusters take items from a queue, so
     // clusters that become resident late simply find less work.
-    SideStream& side = side_stream(st);
-    if (!side.ok) return OCCAM_ERR_CUDA;
-    OCCAM_CUDA(cudaEventRecord(side.fork, st));
-    OCCAM_CUDA(cudaStreamWaitEvent(side.stream, side.fork, 0));
-    // A batch whose every text tile fits as a resident 16-CTA cluster gets
-    // the 16-CTA routing for all of its fused samples (the plan's widening;
-    // a sample that a 16-CTA cluster cannot hold fits no smaller one): its
-    // 8- and 4-CTA launches would have no items, so they are not made.
-    const bool only16 = p.res16 > 0 && (int64_t)b->B * cdiv(b->max_text, 128) <= p.res16;
+    cudaStream_t beside = st;
+    SideStream* side = nullptr;
+    if (!alone) {
+      side = &side_stream(st);
+      if (!side->ok) return OCCAM_ERR_CUDA;
+      OCCAM_CUDA(cudaEventRecord(side->fork, st));
+      OCCAM_CUDA(cudaStreamWaitEvent(side->stream, side->fork, 0));
+      beside = side->stream;
+    }
     Stage2TcParams q8 = q;
     q8.items = p.itemsF8;
     q8.queue = p.counters + CNT_QUEUE8;
     const int ncl8 = fused_launch_clusters(8, L.maxF, sms);
-    if (!only16 && launch_fused(8, mq, mk, mkt, q8, ncl8, side.stream) != 0) return OCCAM_ERR_CUDA;
+    if (!no8 && launch_fused(8, mq, mk, mkt, q8, ncl8, beside) != 0) return OCCAM_ERR_CUDA;
     // samples too large for 8 CTAs: 16-CTA clusters, on this stream ahead of
     // the 4-CTA launch. A launch without items returns at once; it also
     // lets the 8-CTA clusters (larger items) take their SMs first, which
@@ -605,21 +625,25 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     Stage2TcParams q16 = q;
     q16.items = p.itemsF16;
     q16.queue = p.counters + CNT_QUEUE16;
+    q16.pdl = alone && pdl ? 1 : 0;
     const int ncl16 = fused_launch_clusters(16, L.maxF, sms);
     if (launch_fused(16, mq, mk, mkt, q16, ncl16, st) != 0) return OCCAM_ERR_CUDA;
-    // head-split tiles (small batches) meet right behind the 16-CTA launch
-    launch_s2_merge(q16, st);
     // the two-pass kernels (samples the fused kernel cannot hold; often none)
     // follow the 8-CTA launch on the second stream. They are enqueued after
     // the 16-CTA launch: a CTA of theirs takes a whole SM, and enqueued
     // earlier they held every SM before the 16-CTA clusters, which need 16
     // SMs of one GPC, could be placed.
-    OCCAM_TRY(launch_twopass(p, L, sms, b, a, side.stream));
+    if (!no2p) OCCAM_TRY(launch_twopass(p, L, sms, b, a, beside));
     q.queue = p.counters + CNT_QUEUE4;
     const int ncl4 = fused_launch_clusters(4, L.maxF, sms);
-    if (!only16 && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
-    OCCAM_CUDA(cudaEventRecord(side.join, side.stream));
-    OCCAM_CUDA(cudaStreamWaitEvent(st, side.join, 0));
+    if (!no4 && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
+    // head-split tiles (small batches) meet right behind the last fused launch
+    // of this stream
+    launch_s2_merge(q, (int)std::max<int64_t>(1, std::min<int64_t>(max_tiles, kHsMaxTiles)), st);
+    if (side) {
+      OCCAM_CUDA(cudaEventRecord(side->join, side->stream));
+      OCCAM_CUDA(cudaStreamWaitEvent(st, side->join, 0));
+    }
     OCCAM_CUDA(cudaGetLastError());
     trace.mark(st);
   } else {
@@ -980,7 +1004,8 @@ static int prune_impl(const occam_prune_args* args, const occam_prune_out* out, 
     count_launch();
     OCCAM_CUDA(cudaGetLastError());
   }
-  OCCAM_TRY(launch_stage2(b, &a2, L, ws, s2, ref2, args->lambda2, st, trace));
+  // (no trace, no staging copy: the op before Stage II is the finalize kernel)
+  OCCAM_TRY(launch_stage2(b, &a2, L, ws, s2, ref2, args->lambda2, st, trace, !k2_stage && !trace.ev));
   if (args->rule == OCCAM_RULE_BUDGET) {
     // S2 = the budget[b] visual S1 rows with the largest s2 per sample, then
     // the compaction of that mask

@@ -33,12 +33,14 @@ __host__ __device__ inline int s2_stat_splits(int n1, int M) {
   const int s = ((n1 + M + 63) / 64 + 3) / 4;
   return s < 1 ? 1 : s > kStatSplits ? kStatSplits : s;
 }
-// Head split of small batches: when every text tile of the batch fits as
-// kHsGroups resident 16-CTA clusters, each tile's heads are split over that
-// many items; their partial head sums meet in a scratch area of kHsMaxTiles
-// tiles (allocated only when the batch can have no more tiles than that).
-constexpr int kHsMaxTiles = 2;
+// Head split of small batches: where a batch's text tiles leave clusters idle,
+// each tile's heads are split over hsg items (plan_stage2), whose partial head
+// sums meet in a scratch area of kHsSlots slots, one per CTA of those items:
+// slot (tile * hsg + group) * C + rank. It is allocated only for batches of at
+// most kHsMaxTiles samples.
+constexpr int kHsMaxTiles = 18;
 constexpr int kHsGroups = 8;
+constexpr int kHsSlots = 152;
 constexpr int kHsRows = 128;  // text rows of a fused item
 // the fused item's w field: (tile index in the scratch << 8) | (head group << 4) | head groups (0 = 1)
 __host__ __device__ inline int hs_groups(int w) { return (w & 15) ? (w & 15) : 1; }
@@ -121,8 +123,9 @@ struct Stage2Params {
   int4* itemsF8;            // fused items for 8-CTA clusters
   int4* itemsF16;           // fused items for 16-CTA clusters
   int use_fused;            // route eligible samples to the fused tensor-core kernel
-  int res16, res8;          // resident 16- and 8-CTA fused clusters (0: no widening for small batches)
-  int4* itemsHS;            // head-split text tiles (b, j0, slot, head groups), for the merge kernel
+  int res16, res8, res4;    // resident 16-, 8- and 4-CTA fused clusters (0: no widening or splitting for small batches)
+  uint32_t hs_valid;        // bit g: the heads split into g groups of whole key groups, at least 4 heads each
+  int4* itemsHS;            // head-split text tiles (b, j0, slot, head groups | cluster size << 8), for the merge kernel
   int has_ppart;            // the head-split scratch exists
   int32_t* slot_off;        // [B+1] partial-slot range of each sample
   int64_t maxF;
@@ -303,6 +306,7 @@ struct Stage2TcParams {
   float* tau2;
   float lambda2;
   int* status;
+  int pdl;                  // launched with programmatic dependent launch: the prologue overlaps the kernel before it
 };
 
 // stage1.cu
@@ -323,7 +327,7 @@ int launch_stats_tc(const Stage2Params& p, const CUtensorMap& mq128, int grid, c
 
 // stage2_tc.cu
 int fused_resident_clusters(int C);
-void launch_s2_merge(const Stage2TcParams& q, cudaStream_t st);
+void launch_s2_merge(const Stage2TcParams& q, int max_tiles, cudaStream_t st);
 // stage2_scores_tc.cu
 int launch_scores_tc(const Stage2Params& p, const CUtensorMap& mq64, int grid, cudaStream_t st);
 int launch_fused(int C, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mkt, const Stage2TcParams& q,

@@ -22,7 +22,7 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
   // tile of the batch can run at once as a resident 16- (or 8-) CTA cluster,
   // samples take the wider cluster, whose CTAs hold fewer keys and finish
   // each head sooner.
-  int wide = 0, hsg = 1;  // hsg: head groups of a split tile (1: no split)
+  int wide = 0, hsg = 1, hsC = 16;  // hsg: head groups of a split tile (1: no split), of clusters of hsC CTAs
   // the first blockDim.x samples' text lengths and S1 sizes, loaded together
   // up front (one memory round trip instead of two in a row)
   int M0 = 0, n10 = 0;
@@ -37,22 +37,32 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     int total_tiles;
     block_exclusive_scan(tiles, tmp, &total_tiles);
     wide = total_tiles <= p.res16 ? 16 : total_tiles <= p.res8 ? 8 : 0;
-    // head split: a batch of at most kHsMaxTiles tiles whose tiles fit hsg
-    // times over as resident 16-CTA clusters splits each 16-CTA tile's heads
-    // into hsg groups (whole key groups, at least 4 heads each)
-    if (wide == 16 && p.has_ppart && total_tiles <= kHsMaxTiles) {
-      const int grp = p.H / p.Hkv;
-      for (int g = kHsGroups; g >= 2; g >>= 1) {
-        if (total_tiles * g <= p.res16 && p.H % g == 0 && p.H / g >= 4 && (p.H / g) % grp == 0) {
-          hsg = g;
-          break;
-        }
+    // Head split: each tile's heads go to hsg items (whole key groups, at
+    // least 4 heads each), all resident at once. An item's time is its heads
+    // times about 2 us (the chain of one head: MMA, statistics, exchange,
+    // probabilities), on clusters of any size, so 4-CTA clusters (36
+    // resident), where every sample fits them, take the most groups: 8 tiles
+    // of 64 text rows and 540 S1 keys took 77 us on 8-CTA clusters, a head
+    // after the other, and take 33 us and about 8 of merge in 4 groups. One tile has no use for that many, and more than
+    // kHsMaxTiles fill the device unsplit.
+    if (p.has_ppart && total_tiles <= kHsMaxTiles) {
+      // (every sample has a tile, so there are no more samples than threads)
+      const bool fit4 = tid >= p.bt.B || fused_fits(kFusedCluster, n10, M0, p.H);
+      const bool all4 = __syncthreads_and(fit4) && total_tiles > 1;
+      const int res = all4 ? p.res4 : wide == 16 ? p.res16 : 0;
+      // the most groups that divide the heads (hs_valid) and fit at once
+      const uint32_t fits = total_tiles > 0 ? p.hs_valid & ((2u << min(res / total_tiles, kHsGroups)) - 1u) : 0u;
+      if (fits) hsg = 31 - __clz(fits);
+      if (all4 && hsg > 1) {
+        hsC = kFusedCluster;
+        wide = 0;
       }
     }
   }
+  const int hsg4 = hsC == 16 ? 1 : hsg, hsg16 = hsC == 16 ? hsg : 1;  // (1: no split)
   for (int b0 = 0; b0 < p.bt.B; b0 += blockDim.x) {
     const int bb = b0 + tid;
-    int nA = 0, nB = 0, nF = 0, nF8 = 0, nF16 = 0;
+    int nA = 0, nB = 0, tF = 0, nF8 = 0, tF16 = 0;  // (tF, tF16: text tiles, each of hsg4 / hsg16 items)
     if (bb < p.bt.B) {
       const int M = b0 == 0 ? M0 : (int)(p.bt.text_off[bb + 1] - p.bt.text_off[bb]);
       const int n1 = b0 == 0 ? n10 : *((volatile int32_t*)&p.n1[bb]);
@@ -64,11 +74,11 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
       const bool fused8 = w8 || (!w16 && !fused4 && p.use_fused && fused_fits(8, n1, M, p.H));
       const bool fused16 = w16 || (!fused4 && !fused8 && p.use_fused && fused_fits(16, n1, M, p.H));
       if (fused4) {
-        nF = (M + 127) / 128;
+        tF = (M + 127) / 128;
       } else if (fused8) {
         nF8 = (M + 127) / 128;
       } else if (fused16) {
-        nF16 = (M + 127) / 128 * hsg;
+        tF16 = (M + 127) / 128;
       } else {
         const int nch = (n1 + kKeyChunk - 1) / kKeyChunk;
         nA = (M + kStatsTile - 1) / kStatsTile * nhg * s2_stat_splits(n1, M);
@@ -80,12 +90,12 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
         p.tau2[bb] = 0.f;
       }
     }
-    const int nS = nF * kFusedSlotsPerItem + nF8 * kFusedSlotsPerItem8 + nF16 / hsg * kFusedSlotsPerItem16 +
+    const int nS = tF * kFusedSlotsPerItem + nF8 * kFusedSlotsPerItem8 + tF16 * kFusedSlotsPerItem16 +
                    nB;  // s2(r) partial slots of this sample (a split tile's items share its slots)
-    const int nHS = hsg > 1 ? nF16 / hsg : 0;  // this sample's head-split tiles
+    const int nHS = hsg > 1 ? (hsC == 16 ? tF16 : tF) : 0;  // this sample's head-split tiles
     // the seven item and slot counts, scanned together
     __shared__ int mtmp[7 * 33];
-    const int cnt[7] = {nA, nB, nF, nF8, nF16, nS, nHS};
+    const int cnt[7] = {nA, nB, tF * hsg4, nF8, tF16 * hsg16, nS, nHS};
     int ex[7], tot[7];
     block_exclusive_scan_n<7>(cnt, ex, tot, mtmp);
     const int totA = tot[0], totB = tot[1], totF = tot[2], totF8 = tot[3], totF16 = tot[4], totS = tot[5],
@@ -93,19 +103,21 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     const int offA = runA + ex[0], offB = runB + ex[1], offF = runF + ex[2], offF8 = runF8 + ex[3],
               offF16 = runF16 + ex[4], offS = runS + ex[5], offHS = runHS + ex[6];
     if (bb < p.bt.B) {
-      for (int i = 0; i < nF; ++i)
-        if (offF + i < p.maxF) p.itemsF[offF + i] = make_int4(bb, i * 128, offS + i * kFusedSlotsPerItem, 0);
+      // a tile's items: one, or its head groups in turn
+      auto tile_items = [&](int4* items, int off, int tiles, int g_n, int slots) {
+        for (int t = 0; t < tiles; ++t)
+          for (int g = 0; g < g_n; ++g, ++off)
+            if (off < p.maxF)
+              items[off] = make_int4(bb, t * 128, offS + t * slots, g_n > 1 ? ((offHS + t) << 8) | (g << 4) | g_n : 0);
+      };
+      tile_items(p.itemsF, offF, tF, hsg4, kFusedSlotsPerItem);
+      tile_items(p.itemsF16, offF16, tF16, hsg16, kFusedSlotsPerItem16);
       for (int i = 0; i < nF8; ++i)
         if (offF8 + i < p.maxF) p.itemsF8[offF8 + i] = make_int4(bb, i * 128, offS + i * kFusedSlotsPerItem8, 0);
-      for (int i = 0; i < nF16; ++i) {
-        const int tile = i / hsg, hg = i % hsg;
-        const int w = hsg > 1 ? ((offHS + tile) << 8) | (hg << 4) | hsg : 0;
-        if (offF16 + i < p.maxF)
-          p.itemsF16[offF16 + i] = make_int4(bb, tile * 128, offS + tile * kFusedSlotsPerItem16, w);
-      }
       for (int t = 0; t < nHS; ++t)
         if (offHS + t < kHsMaxTiles)
-          p.itemsHS[offHS + t] = make_int4(bb, t * 128, offS + t * kFusedSlotsPerItem16, hsg);
+          p.itemsHS[offHS + t] = make_int4(
+              bb, t * 128, offS + t * (hsC == 16 ? kFusedSlotsPerItem16 : kFusedSlotsPerItem), hsg | (hsC << 8));
       p.itemA_off[bb] = offA;
       p.itemB_off[bb] = offB;
       p.slot_off[bb] = offS;

@@ -486,6 +486,9 @@ __global__ void __launch_bounds__(256) stage1_finalize_kernel(Stage1FinalizePara
       ++pos;
     }
   }
+  // the fused Stage II may start its prologue (a launch that does waits for
+  // the plan before it reads any of this kernel's results)
+  pdl_trigger();
   if (!p.do_plan) return;
   // the last CTA to finish plans Stage II
   __threadfence();

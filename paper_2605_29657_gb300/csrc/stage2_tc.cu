@@ -331,12 +331,14 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
   Smem<C>& sm = *reinterpret_cast<Smem<C>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = (int)tc::cluster_rank();
-  const int nF = p.counters[C == 16 ? CNT_NF16 : C == 8 ? CNT_NF8 : CNT_NF];
+  int nF = p.pdl ? 0x7fffffff : p.counters[C == 16 ? CNT_NF16 : C == 8 ? CNT_NF8 : CNT_NF];
   // no work for this cluster (every CTA of every cluster reads the same
   // count): leave before touching shared memory, TMEM or the cluster. With
   // nF items, the clusters numbered nF and up can never be handed one (at
   // most nF hand-outs succeed and the first nF clusters keep drawing until
-  // the queue is empty), so they leave too, freeing their SMs at once.
+  // the queue is empty), so they leave too, freeing their SMs at once. (A
+  // programmatic dependent launch does not know yet: its prologue overlaps
+  // the end of the plan, and the count is read behind it.)
   if ((int)blockIdx.x / C >= nF) return;
   volatile int* abort = &sm.abort;
 
@@ -380,6 +382,10 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
   tc::fence_after();
   // peers' barriers must be initialised before anyone stores into them remotely
   tc::cluster_sync_all();
+  if (p.pdl) {
+    pdl_wait();
+    nF = *(volatile int*)&p.counters[C == 16 ? CNT_NF16 : C == 8 ? CNT_NF8 : CNT_NF];
+  }
   const uint32_t tmem = sm.tmem_base;
   const int H = p.H;
 
@@ -701,8 +707,8 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
       if (g.nhg > 1) {
         // a head group of a split tile: its partial head sums go to the
         // scratch, rows of zeros past the text; the merge kernel reduces them
-        float* dst = p.ppart + ((((int64_t)g.hs_tile * kHsGroups + hs_group(p.items[item].w)) * 16 + rank) * kHsRows + j) *
-                                   PMAX;
+        float* dst =
+            p.ppart + ((((int64_t)g.hs_tile * g.nhg + hs_group(p.items[item].w)) * C + rank) * kHsRows + j) * PMAX;
 #pragma unroll
         for (int q = 0; q < NPC; ++q) {
           if (q < npi) {
@@ -811,8 +817,7 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
   tc::cluster_sync_all();
 }
 
-// Merge of head-split tiles. CTA (t, rank) of a kHsMaxTiles x 16 grid takes
-// tile t's S1 keys of cluster rank `rank`: key column k and row quarter q
+// Merge of head-split tiles. CTA (t, rank) of a tiles x 16 grid takes tile t's S1 keys of cluster rank `rank`: key column k and row quarter q
 // belong to thread q * kFusedMaxOwnImg + k. A thread sums the head groups'
 // partials (in group order) for each of its rows (rows q, q + 4, ...), with
 // every load of its rows issued before the adds, and keeps their max and
@@ -832,8 +837,10 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
   const int t = blockIdx.x / 16, rank = blockIdx.x % 16;
   if (t >= p.counters[CNT_NHS]) return;
   const int4 it = p.itemsHS[t];
-  const int nhg = it.w;
-  const ItemGeom g = item_geom<16>(p, make_int4(it.x, it.y, it.z, 0), rank);
+  const int nhg = it.w & 255, C = it.w >> 8;
+  if (rank >= C) return;
+  const int4 whole = make_int4(it.x, it.y, it.z, 0);
+  const ItemGeom g = C == 16 ? item_geom<16>(p, whole, rank) : item_geom<kFusedCluster>(p, whole, rank);
   const int k = threadIdx.x % kFusedMaxOwnImg, q = threadIdx.x / kFusedMaxOwnImg, lane = threadIdx.x & 31;
   const int rows = min(kHsRows, g.M - g.j0);
   const float invH = 1.0f / (float)p.H;
@@ -849,7 +856,7 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
   pdl_wait();
   float cmax = 0.f, rsum = 0.f;
   if (k < g.own_img) {
-    const float* src = p.ppart + (((int64_t)t * kHsGroups * 16 + rank) * kHsRows) * PMAX + k;
+    const float* src = p.ppart + (((int64_t)t * nhg * C + rank) * kHsRows) * PMAX + k;
     // this thread's rows q, q + 4, ..., up to eight at a time with every
     // group's load in flight before the adds; sums in group order, then row
     // order
@@ -860,7 +867,7 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
 #pragma unroll
         for (int hg = 0; hg < kHsGroups; ++hg) {
           const int r = r0 + u * kMergeQ;
-          v[u][hg] = (r < rows && hg < nhg) ? __ldcg(src + ((int64_t)hg * 16 * kHsRows + r) * PMAX) : 0.f;
+          v[u][hg] = (r < rows && hg < nhg) ? __ldcg(src + ((int64_t)hg * C * kHsRows + r) * PMAX) : 0.f;
         }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -923,13 +930,13 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
   }
 }
 
-void launch_s2_merge(const Stage2TcParams& q, cudaStream_t st) {
+void launch_s2_merge(const Stage2TcParams& q, int max_tiles, cudaStream_t st) {
   if (q.ppart) {
-    // launched right behind the 16-CTA fused kernel with programmatic
+    // launched right behind the last fused kernel of its stream with programmatic
     // stream serialization: its item, geometry and key-row loads overlap the
     // end of that kernel, and it waits for the partials (pdl_wait)
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kHsMaxTiles * 16);
+    cfg.gridDim = dim3(max_tiles * 16);
     cfg.blockDim = dim3(kMergeThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -983,13 +990,15 @@ int launch_fused(int C, const CUtensorMap& mq, const CUtensorMap& mk, const CUte
   cfg.blockDim = dim3(s2f::THREADS);
   cfg.dynamicSmemBytes = s2_fused_smem_bytes(C);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = q.pdl ? 2 : 1;
   // the register split inside the kernel needs the launch to reserve at least
   // REG_NEEDED registers per CTA; refuse rather than launch a kernel whose
   // setmaxnreg.inc could never be satisfied
