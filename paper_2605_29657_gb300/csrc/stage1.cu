@@ -30,29 +30,31 @@ struct Geo {
   static constexpr int kRowBytes = H * D * 2;   // 2048 / 2304 / 4096 for d1 = 64 / 72 / 128
   static constexpr int kStageBytes = kTileRows * kRowBytes;
   static constexpr int kSmem = kStages * kStageBytes + 64;
-  static constexpr int kLaneDims = D / 8;       // dims of one (row, head) per lane (8 lanes share it)
+  // d1 = 72: a thread takes a whole (row, head), nine 16-byte loads 144 bytes
+  // apart from its neighbours' (an odd number of 16-byte units: no bank
+  // conflicts). Otherwise, where that stride would put all lanes on the same
+  // banks, 8 lanes share a (row, head), D / 8 dims each. (Shared by 8 lanes,
+  // the 18-byte slices of d1 = 72 took nine 2-byte loads each: 38 us for
+  // 158 MB of keys, against 30 now.)
+  static constexpr bool kWhole = D == 72;
+  static constexpr int kLaneDims = kWhole ? D : D / 8;  // dims of one (row, head) per lane
   static_assert(D % 8 == 0 && kRowBytes % 16 == 0, "rows in whole 16-byte units");
 };
 static_assert(Geo<128>::kSmem <= 227 * 1024, "shared memory per CTA");
 
-// n consecutive bf16 values as floats: 16-byte loads when the lane's slice is
-// a whole number of them, else 2-byte loads (d1 = 72: 9 dims = 18 bytes)
+// N consecutive bf16 values as floats, in 16-byte loads
 template <int N>
 __device__ __forceinline__ void load_bf16(const unsigned char* src, float (&out)[N]) {
-  if constexpr (N % 8 == 0) {
+  static_assert(N % 8 == 0, "whole 16-byte loads");
 #pragma unroll
-    for (int c = 0; c < N / 8; ++c) {
-      const uint4 raw = *reinterpret_cast<const uint4*>(src + 16 * c);
-      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  for (int c = 0; c < N / 8; ++c) {
+    const uint4 raw = *reinterpret_cast<const uint4*>(src + 16 * c);
+    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        out[8 * c + 2 * i] = bf16_lo(w[i]);
-        out[8 * c + 2 * i + 1] = bf16_hi(w[i]);
-      }
+    for (int i = 0; i < 4; ++i) {
+      out[8 * c + 2 * i] = bf16_lo(w[i]);
+      out[8 * c + 2 * i + 1] = bf16_hi(w[i]);
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(src)[i] << 16);
   }
 }
 }  // namespace cls
@@ -85,10 +87,14 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
   // lane layout for the dot products: 8 lanes share one (row, head); lane
   // k = lane & 7 owns dims [k D/8, (k+1) D/8) of that head. The four (row,
   // head) slots of a warp share one row, so segment changes are warp-uniform.
-  const int slot = warp * 4 + (lane >> 3);   // 0..31
+  // With whole (row, head) pairs per thread the tile is one step, thread t
+  // taking head t & 15 of row t >> 4.
+  constexpr bool kWhole = Geo<D>::kWhole;
+  constexpr int kSteps = kWhole ? 1 : kTileRows / 2;
+  const int slot = kWhole ? tid : warp * 4 + (lane >> 3);  // 0..31 (0..255)
   const int my_h = slot & (H - 1);
-  const int my_rr = slot >> 4;               // 0..1: row parity inside a step
-  const int kv = lane & 7;
+  const int my_rr = slot >> 4;               // 0..1: row parity inside a step (0..15: row of the tile)
+  const int kv = kWhole ? 0 : lane & 7;
   int64_t seg_lo = 0, seg_hi = 0;            // rows of the segment q belongs to
   float q[NL];
 
@@ -109,7 +115,7 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
     const int64_t r0 = (t0 + it) * kTileRows;
     const int rows = (int)min((int64_t)kTileRows, R - r0);
 #pragma unroll
-    for (int step = 0; step < kTileRows / 2; ++step) {
+    for (int step = 0; step < kSteps; ++step) {
       const int rr = step * 2 + my_rr;
       const int64_t row = r0 + rr;
       float acc = 0.f;
@@ -121,14 +127,29 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
           seg_hi = p.bt.seg_off[sg + 1];
           load_bf16<NL>(reinterpret_cast<const unsigned char*>(p.q_cls + ((int64_t)sg * H + my_h) * D + kv * NL), q);
         }
-        float kx[NL];
-        load_bf16<NL>(buf + rr * kRowBytes + my_h * D * 2 + kv * NL * 2, kx);
+        if constexpr (kWhole) {
+          // eight partial sums of nine terms, then a tree
+          float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int i = 0; i < NL; ++i) acc = fmaf(q[i], kx[i], acc);
+          for (int c = 0; c < D / 8; ++c) {
+            float kx[8];
+            load_bf16<8>(buf + rr * kRowBytes + my_h * D * 2 + 16 * c, kx);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a8[i] = fmaf(q[8 * c + i], kx[i], a8[i]);
+          }
+          acc = ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
+        } else {
+          float kx[NL];
+          load_bf16<NL>(buf + rr * kRowBytes + my_h * D * 2 + kv * NL * 2, kx);
+#pragma unroll
+          for (int i = 0; i < NL; ++i) acc = fmaf(q[i], kx[i], acc);
+        }
       }
-      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+      if constexpr (!kWhole) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+      }
       if (kv == 0 && rr < rows) p.logits[row * H + my_h] = acc * p.scale;  // log2 units
     }
     __syncthreads();
