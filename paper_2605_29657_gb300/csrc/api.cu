@@ -891,7 +891,7 @@ int occam_score_stage2(const occam_batch* batch, const occam_stage2_args* args, 
   OCCAM_TRY(check_ws(batch, 1, args->H2, workspace, workspace_bytes, &L));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   set_smem_attrs();
-  OCCAM_TRY(mark_roles(batch, L, workspace, st));
+  // (the finalize kernel writes the row roles)
   OCCAM_CUDA(cudaMemsetAsync(at<unsigned char>(workspace, L.zero_begin), 0, L.zero_end - L.zero_begin, st));
   OCCAM_CUDA(cudaMemsetAsync(s2, 0, batch->total_rows * 4, st));
   // S1 lists from the given mask (registers always in S1) and the Stage-II plan
