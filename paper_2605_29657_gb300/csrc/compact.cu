@@ -591,8 +591,8 @@ __global__ void __launch_bounds__(1024) l2_finish_kernel(Lambda2Params p) {
 }
 
 // The same selection by one cluster of 16 CTAs, for up to kL2ClusterRows rows:
-// CTA r takes the r-th sixteenth of the rows and keeps their keys in shared
-// memory, so each digit costs a pass over shared memory, the sums of the
+// CTA r takes the r-th sixteenth of the rows and keeps its candidates' keys in
+// shared memory, so each digit costs a pass over shared memory, the sums of the
 // buckets over the cluster (distributed shared memory), the choice in CTA 0
 // and three cluster barriers. Bound by that chain; the grid-wide
 // kernels above pay a launch per step (74 us a call on 185,600 rows).
@@ -608,6 +608,7 @@ struct L2Shared {
   float ref[kL2Staged];
   unsigned long long kept[2 * kL2Window + 1];
   int n, cnt;
+  int rows;  // this CTA's candidate rows
   float min_ref;  // CTA 0: the smallest positive reference
   // written by CTA 0 into every CTA
   uint32_t prefix;
@@ -617,7 +618,7 @@ struct L2Shared {
 }  // namespace
 
 __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p) {
-  extern __shared__ uint32_t l2_keys[];
+  extern __shared__ uint32_t l2_keys[];  // [chunk] the candidates' keys, then [chunk] their rows of the chunk
   __shared__ L2Shared sm;
   namespace cg = cooperative_groups;
   const cg::cluster_group cluster = cg::this_cluster();
@@ -627,6 +628,7 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
   const int64_t chunk = (R + kL2ClusterCtas - 1) / kL2ClusterCtas;
   const int64_t c0 = min(R, rank * chunk), c1 = min(R, c0 + chunk);
   const int n = (int)(c1 - c0);
+  uint16_t* const l2_idx = reinterpret_cast<uint16_t*>(l2_keys + chunk);
   const bool staged = p.bt.B <= kL2Staged;
   constexpr int NW = 2 * kL2Window + 1;
   for (int i = tid; i < 3 * kL2Digits; i += kL2Threads) (&sm.hist[0][0])[i] = 0;
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
   }
   if (tid < NW) sm.kept[tid] = 0;
   if (tid == 0) {
-    sm.n = sm.cnt = 0;
+    sm.n = sm.cnt = sm.rows = 0;
     sm.done = 0;
   }
   __syncthreads();
@@ -664,43 +666,65 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
   cluster.sync();
   const int64_t* ro = staged ? sm.ro : p.bt.row_off;
   const float* ref2 = staged ? sm.ref : p.ref2;
-  // keys, and the histogram of their top digit; eight rows' loads and sample
-  // searches at once per thread
+  // the candidates' rows (any order), compacted: the divisions and searches
+  // below, 16 SMs' bound over all rows, are then for candidates alone
+  for (int i0 = tid & ~31; i0 < n; i0 += 16 * kL2Threads) {  // (whole warps)
+    bool c[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = i0 + (tid & 31) + u * kL2Threads;
+      c[u] = i < n && p.keep1[c0 + i] != 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = i0 + (tid & 31) + u * kL2Threads;
+      const bool on = c[u] && !test_bit(sm.regs, i);
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      int at = 0;
+      if ((tid & 31) == 0 && m) at = atomicAdd(&sm.rows, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << (tid & 31)) - 1u));
+      if (on) l2_idx[at] = (uint16_t)i;
+    }
+  }
+  __syncthreads();
+  const int rows = sm.rows;
+  // their keys (0 where the sample's reference is not positive), and the
+  // histogram of the top digit
   int cand = 0;
   int steps = 0;
   while ((1 << steps) < p.bt.B) ++steps;
-  for (int i0 = tid; i0 < n; i0 += 8 * kL2Threads) {
-    float s[8];
-    bool c[8];
-    int lo[8];
+  for (int i0 = tid; i0 < rows; i0 += 4 * kL2Threads) {
+    float s[4];
+    int64_t r[4];
+    int lo[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * kL2Threads;
-      s[u] = i < n ? p.s2[c0 + i] : 0.f;
-      c[u] = i < n && p.keep1[c0 + i] != 0;
+      r[u] = i < rows ? c0 + l2_idx[i] : -1;
+      s[u] = i < rows ? p.s2[r[u]] : 0.f;
       lo[u] = 0;
     }
     // the largest b with ro[b] <= row
     for (int h = steps - 1; h >= 0; --h) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
+      for (int u = 0; u < 4; ++u) {
         const int b = lo[u] + (1 << h);
-        if (b < p.bt.B && ro[b] <= c0 + i0 + u * kL2Threads) lo[u] = b;
+        if (b < p.bt.B && ro[b] <= r[u]) lo[u] = b;
       }
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * kL2Threads;
-      uint32_t key = 0;
-      if (c[u] && !test_bit(sm.regs, i)) {
+      if (i < rows) {
         const float ref = ref2[lo[u]];
+        uint32_t key = 0;
         if (ref > 0.f) {
           key = 0x80000000u | __float_as_uint(__fdiv_rn(s[u], ref));
           ++cand;
           atomicAdd(&sm.hist[0][key >> 21], 1u);
         }
+        l2_keys[i] = key;
       }
-      if (i < n) l2_keys[i] = key;
     }
   }
   cand = __reduce_add_sync(0xffffffffu, cand);
@@ -709,7 +733,7 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
     if (level > 0) {
       const uint32_t prefix = sm.prefix, mask = l2_mask_above(level);
       const int shift = l2_shift(level);
-      for (int i = tid; i < n; i += kL2Threads) {
+      for (int i = tid; i < rows; i += kL2Threads) {
         const uint32_t key = l2_keys[i];
         if ((key >> 31) && (key & mask) == prefix) atomicAdd(&sm.hist[level][(key >> shift) & (kL2Digits - 1)], 1u);
       }
@@ -775,7 +799,7 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
   const bool margin = lam0 > 1e-30f && lam0 * root->min_ref > 1e-30f;
   auto kept_at = [&](const float* lam, int* c, auto count) {
     const float first = lam[0], last = lam[decltype(count)::value - 1];
-    for (int i = tid; i < n; i += kL2Threads) {
+    for (int i = tid; i < rows; i += kL2Threads) {
       const uint32_t key = l2_keys[i];
       if (key >> 31) {
         const int q = (int)(key & 0x7fffffffu);
@@ -785,7 +809,7 @@ __global__ void __launch_bounds__(kL2Threads) l2_cluster_kernel(Lambda2Params p)
           for (int j = 0; j < decltype(count)::value; ++j) ++c[j];
           continue;
         }
-        const int64_t r = c0 + i;
+        const int64_t r = c0 + l2_idx[i];
         const float s = p.s2[r], ref = ref2[upper_interval(ro, p.bt.B, r)];
 #pragma unroll
         for (int j = 0; j < decltype(count)::value; ++j) c[j] += s >= __fmul_rn(lam[j], ref) ? 1 : 0;
@@ -849,7 +873,7 @@ int launch_l2_cluster(const Lambda2Params& p, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kL2ClusterCtas);
   cfg.blockDim = dim3(kL2Threads);
-  cfg.dynamicSmemBytes = (size_t)chunk * 4;
+  cfg.dynamicSmemBytes = (size_t)chunk * 6;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -860,7 +884,7 @@ int launch_l2_cluster(const Lambda2Params& p, cudaStream_t st) {
   cfg.numAttrs = 1;
   if (cudaFuncSetAttribute(l2_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
       cudaFuncSetAttribute(l2_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(kL2ClusterRows / kL2ClusterCtas * 4)) != cudaSuccess)
+                           (int)(kL2ClusterRows / kL2ClusterCtas * 6)) != cudaSuccess)
     return 1;
   count_launch();
   return cudaLaunchKernelEx(&cfg, l2_cluster_kernel, p) == cudaSuccess ? 0 : 1;

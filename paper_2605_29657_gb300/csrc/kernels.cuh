@@ -253,7 +253,7 @@ constexpr int kL2Window = 4;            // fp32 steps either way whose kept coun
 // up to this many rows lambda2 is selected by one cluster of 16 CTAs that
 // keeps every row's key in shared memory; above, by grid-wide passes
 constexpr int kL2ClusterCtas = 16;
-constexpr int64_t kL2ClusterRows = (int64_t)kL2ClusterCtas * 40960;
+constexpr int64_t kL2ClusterRows = (int64_t)kL2ClusterCtas * 28672;  // (6 bytes a row beside 48 KB of histograms and offsets)
 constexpr int kL2SelBytes = 32 * 1024;  // workspace scratch of the selection
 
 // mean-threshold reference (component ablation): ref[u] = mean of s over the

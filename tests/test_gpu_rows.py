@@ -114,8 +114,8 @@ def test_construct_registers_several_windows():
     ([17, 1, 300], [1, 2]),
     ([3] * 1200, [2] * 600),                     # more samples than are staged
     ([100000, 227680], [1, 1]),
-    ([655360], [1]),                             # the most rows of the one-cluster kernel
-    ([655361], [1]),                             # the grid-wide kernels
+    ([458752], [1]),                             # the most rows of the one-cluster kernel
+    ([458753], [1]),                             # the grid-wide kernels
 ])
 def test_calibrate_lambda2_row_ranges(seg_rows, segs):
     import paper_2605_29657_gb300 as occ
