@@ -481,6 +481,12 @@ int launch_twopass(const Stage2Params& p, const WsLayout& L, int sms, const occa
   return OCCAM_OK;
 }
 
+// Samples that a 16-CTA cluster holds with all their rows in S1 take no
+// two-pass kernels.
+bool no_twopass(const occam_batch* b, const occam_stage2_args* a) {
+  return fused_fits(16, b->max_sample_rows, b->max_text, a->H2);
+}
+
 // Stage-II parameter block (the same for the plan, built by the Stage-I
 // finalize kernel, and for the Stage-II kernels).
 Stage2Params stage2_params(const occam_batch* b, const occam_stage2_args* a, const WsLayout& L, void* ws, float* s2,
@@ -520,6 +526,11 @@ Stage2Params stage2_params(const occam_batch* b, const occam_stage2_args* a, con
   p.itemsHS = at<int4>(ws, L.itemsHS);
   p.has_ppart = L.ppart != 0 ? 1 : 0;
   p.res8 = widening_enabled() ? fused_resident_clusters(8) : 0;
+  // A batch whose every tile fits as a resident 16-CTA cluster needs the 8-CTA
+  // launch for split tiles alone: not with one tile, and not where samples
+  // may need the two-pass kernels, which it would delay on their stream.
+  const int64_t max_tiles = (int64_t)b->B * cdiv(b->max_text, 128);
+  p.split8 = !(p.res16 > 0 && max_tiles <= p.res16) || (max_tiles > 1 && p.has_ppart && no_twopass(b, a)) ? 1 : 0;
   p.hs_valid = 0;
   for (int g = 2; g <= kHsGroups; ++g)
     if (a->H2 % g == 0 && a->H2 / g >= 4 && (a->H2 / g) % (a->H2 / p.Hkv) == 0) p.hs_valid |= 1u << g;
@@ -586,20 +597,19 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     q.status = p.status;
     // A batch whose every text tile fits as a resident 16-CTA cluster takes
     // 16-CTA clusters for all of its fused samples (the plan's widening; a
-    // sample that a 16-CTA cluster cannot hold fits no smaller one) or, with
-    // more than one tile, 4-CTA clusters with split heads: a launch that can
-    // have no items is not made.
+    // sample that a 16-CTA cluster cannot hold fits no smaller one), unless
+    // it has more than one tile and the plan splits their heads over 4- and
+    // 8-CTA clusters: launches that can have no items are not made.
     const int64_t max_tiles = (int64_t)b->B * cdiv(b->max_text, 128);
-    const bool no8 = p.res16 > 0 && max_tiles <= p.res16;
-    const bool no4 = no8 && (max_tiles == 1 || !q.ppart);
-    // Samples that a 16-CTA cluster holds with all their rows in S1 take no
-    // two-pass kernels.
-    const bool no2p = fused_fits(16, b->max_sample_rows, b->max_text, a->H2);
+    const bool only16 = p.res16 > 0 && max_tiles <= p.res16 && (max_tiles == 1 || !q.ppart);
+    const bool no2p = no_twopass(b, a);
     // With the 16-CTA launch alone (one text tile) nothing runs beside it: no
     // second stream, and it follows the finalize kernel with programmatic
     // dependent launch.
-    const bool alone = no4 && no2p;
+    const bool alone = only16 && no2p;
     q.pdl = 0;
+    q.merge8 = 0;
+    const int merge_tiles = (int)std::max<int64_t>(1, std::min<int64_t>(max_tiles, kHsMaxTiles));
     // The 8-CTA launch runs beside the 4-CTA one on a second stream (fork and
     // join by events), so SMs one of them leaves idle serve the other. Both
     // launch a cluster per SM group; clusters take items from a queue, so
@@ -617,7 +627,13 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     q8.items = p.itemsF8;
     q8.queue = p.counters + CNT_QUEUE8;
     const int ncl8 = fused_launch_clusters(8, L.maxF, sms);
-    if (!no8 && launch_fused(8, mq, mk, mkt, q8, ncl8, beside) != 0) return OCCAM_ERR_CUDA;
+    if (p.split8) {
+      if (launch_fused(8, mq, mk, mkt, q8, ncl8, beside) != 0) return OCCAM_ERR_CUDA;
+      // head-split tiles (small batches) meet right behind the fused launches
+      // of their stream
+      q8.merge8 = 1;
+      launch_s2_merge(q8, merge_tiles, beside);
+    }
     // samples too large for 8 CTAs: 16-CTA clusters, on this stream ahead of
     // the 4-CTA launch. A launch without items returns at once; it also
     // lets the 8-CTA clusters (larger items) take their SMs first, which
@@ -636,10 +652,8 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     if (!no2p) OCCAM_TRY(launch_twopass(p, L, sms, b, a, beside));
     q.queue = p.counters + CNT_QUEUE4;
     const int ncl4 = fused_launch_clusters(4, L.maxF, sms);
-    if (!no4 && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
-    // head-split tiles (small batches) meet right behind the last fused launch
-    // of this stream
-    launch_s2_merge(q, (int)std::max<int64_t>(1, std::min<int64_t>(max_tiles, kHsMaxTiles)), st);
+    if (!only16 && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
+    launch_s2_merge(q, merge_tiles, st);
     if (side) {
       OCCAM_CUDA(cudaEventRecord(side->join, side->stream));
       OCCAM_CUDA(cudaStreamWaitEvent(st, side->join, 0));

@@ -35,17 +35,16 @@ __host__ __device__ inline int s2_stat_splits(int n1, int M) {
 }
 // Head split of small batches: where a batch's text tiles leave clusters idle,
 // each tile's heads are split over hsg items (plan_stage2), whose partial head
-// sums meet in a scratch area of kHsSlots slots, one per CTA of those items:
-// slot (tile * hsg + group) * C + rank. It is allocated only for batches of at
-// most kHsMaxTiles samples.
+// sums meet in a scratch area of kHsSlots slots, one per CTA of those items.
+// It is allocated only for batches of at most kHsMaxTiles samples.
 constexpr int kHsMaxTiles = 18;
 constexpr int kHsGroups = 8;
 constexpr int kHsSlots = 152;
 constexpr int kHsRows = 128;  // text rows of a fused item
-// the fused item's w field: (tile index in the scratch << 8) | (head group << 4) | head groups (0 = 1)
+// the fused item's w field: (scratch slot of its first CTA << 8) | (head group << 4) | head groups (0 = 1)
 __host__ __device__ inline int hs_groups(int w) { return (w & 15) ? (w & 15) : 1; }
 __host__ __device__ inline int hs_group(int w) { return (w >> 4) & 15; }
-__host__ __device__ inline int hs_tile(int w) { return w >> 8; }
+__host__ __device__ inline int hs_slot(int w) { return w >> 8; }
 constexpr int kFusedSlotsPerItem = kFusedCluster * kFusedPartialWarps;  // s2(r) partials per C=4 item
 constexpr int kFusedSlotsPerItem8 = 8 * kFusedPartialWarps;             // and per C=8 item
 constexpr int kFusedSlotsPerItem16 = 16 * kFusedPartialWarps;           // and per C=16 item
@@ -124,8 +123,9 @@ struct Stage2Params {
   int4* itemsF16;           // fused items for 16-CTA clusters
   int use_fused;            // route eligible samples to the fused tensor-core kernel
   int res16, res8, res4;    // resident 16-, 8- and 4-CTA fused clusters (0: no widening or splitting for small batches)
+  int split8;               // the 8-CTA launch is made and may take split tiles
   uint32_t hs_valid;        // bit g: the heads split into g groups of whole key groups, at least 4 heads each
-  int4* itemsHS;            // head-split text tiles (b, j0, slot, head groups | cluster size << 8), for the merge kernel
+  int4* itemsHS;            // head-split text tiles (b, j0, slot, head groups | cluster size << 8 | first scratch slot << 16), for the merge kernel
   int has_ppart;            // the head-split scratch exists
   int32_t* slot_off;        // [B+1] partial-slot range of each sample
   int64_t maxF;
@@ -306,6 +306,7 @@ struct Stage2TcParams {
   float* tau2;
   float lambda2;
   int* status;
+  int merge8;               // merge kernel: take the tiles of 8-CTA clusters (else those of the others)
   int pdl;                  // launched with programmatic dependent launch: the prologue overlaps the kernel before it
 };
 

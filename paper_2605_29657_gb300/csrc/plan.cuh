@@ -17,12 +17,12 @@ namespace occam {
 __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
   const int tid = threadIdx.x;
   const int nhg = (p.H + kHeadGroup - 1) / kHeadGroup;
-  int runA = 0, runB = 0, runF = 0, runF8 = 0, runF16 = 0, runS = 0, runHS = 0;
+  int runA = 0, runB = 0, runF = 0, runF8 = 0, runF16 = 0, runS = 0, runHS = 0, runP = 0;
   // A small batch leaves most SMs idle with 4-CTA clusters: when every text
   // tile of the batch can run at once as a resident 16- (or 8-) CTA cluster,
   // samples take the wider cluster, whose CTAs hold fewer keys and finish
   // each head sooner.
-  int wide = 0, hsg = 1, hsC = 16;  // hsg: head groups of a split tile (1: no split), of clusters of hsC CTAs
+  int wide = 0, hsg = 1, hs16 = 1;  // hsg: head groups of a split tile (1: no split), on 16-CTA clusters or on 4 and 8
   // the first blockDim.x samples' text lengths and S1 sizes, loaded together
   // up front (one memory round trip instead of two in a row)
   int M0 = 0, n10 = 0;
@@ -31,38 +31,58 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     n10 = *((volatile int32_t*)&p.n1[tid]);
   }
   if (p.use_fused) {
+    // the batch's text tiles and, for one that may split its heads, the CTAs
+    // that one group of every tile takes (in the high bits; a sample's tiles
+    // count as 100 at most, far above any rule)
     int tiles = 0;
-    for (int b = tid; b < p.bt.B; b += blockDim.x)
-      tiles += b == tid ? (M0 + 127) / 128 : (int)((p.bt.text_off[b + 1] - p.bt.text_off[b] + 127) / 128);
-    int total_tiles;
+    bool fit = true;
+    if (p.has_ppart) {  // (at most kHsMaxTiles samples)
+      if (tid < p.bt.B) {
+        const bool fit4 = fused_fits(kFusedCluster, n10, M0, p.H);
+        fit = fit4 || (p.split8 && fused_fits(8, n10, M0, p.H));
+        tiles = min((M0 + 127) / 128, 100);
+        tiles |= tiles * (fit4 ? kFusedCluster : 8) << 12;
+      }
+    } else {
+      for (int b = tid; b < p.bt.B; b += blockDim.x)
+        tiles += b == tid ? (M0 + 127) / 128 : (int)((p.bt.text_off[b + 1] - p.bt.text_off[b] + 127) / 128);
+    }
+    int total_tiles, ctas = 0;
     block_exclusive_scan(tiles, tmp, &total_tiles);
+    if (p.has_ppart) {
+      ctas = total_tiles >> 12;
+      total_tiles &= 4095;
+    }
     wide = total_tiles <= p.res16 ? 16 : total_tiles <= p.res8 ? 8 : 0;
     // Head split: each tile's heads go to hsg items (whole key groups, at
     // least 4 heads each), all resident at once. An item's time is its heads
     // times about 2 us (the chain of one head: MMA, statistics, exchange,
-    // probabilities), on clusters of any size, so 4-CTA clusters (36
-    // resident), where every sample fits them, take the most groups: 8 tiles
-    // of 64 text rows and 540 S1 keys took 77 us on 8-CTA clusters, a head
-    // after the other, and take 33 us and about 8 of merge in 4 groups. One tile has no use for that many, and more than
+    // probabilities), on clusters of any size, so the smallest clusters, 4
+    // CTAs (36 resident) or 8 for the samples that do not fit those, take the
+    // most groups: 8 tiles of 64 text rows and 540 S1 keys took 77 us on
+    // 8-CTA clusters, a head after the other, and take 33 us and about 8 of
+    // merge in 4 groups. One tile has no use for that many, and more than
     // kHsMaxTiles fill the device unsplit.
     if (p.has_ppart && total_tiles <= kHsMaxTiles) {
-      // (every sample has a tile, so there are no more samples than threads)
-      const bool fit4 = tid >= p.bt.B || fused_fits(kFusedCluster, n10, M0, p.H);
-      const bool all4 = __syncthreads_and(fit4) && total_tiles > 1;
-      const int res = all4 ? p.res4 : wide == 16 ? p.res16 : 0;
+      const bool small = __syncthreads_and(fit) && total_tiles > 1 && p.res4 > 0;
       // the most groups that divide the heads (hs_valid) and fit at once
-      const uint32_t fits = total_tiles > 0 ? p.hs_valid & ((2u << min(res / total_tiles, kHsGroups)) - 1u) : 0u;
+      int most = 0;
+      if (small)
+        most = p.res4 * kFusedCluster / ctas;
+      else if (wide == 16 && total_tiles > 0)
+        most = p.res16 / total_tiles;
+      const uint32_t fits = p.hs_valid & ((2u << min(most, kHsGroups)) - 1u);
       if (fits) hsg = 31 - __clz(fits);
-      if (all4 && hsg > 1) {
-        hsC = kFusedCluster;
+      if (small && hsg > 1) {
+        hs16 = 0;
         wide = 0;
       }
     }
   }
-  const int hsg4 = hsC == 16 ? 1 : hsg, hsg16 = hsC == 16 ? hsg : 1;  // (1: no split)
+  const int hsg4 = hs16 ? 1 : hsg, hsg16 = hs16 ? hsg : 1;  // of tiles on 4- and 8-, and on 16-CTA clusters (1: no split)
   for (int b0 = 0; b0 < p.bt.B; b0 += blockDim.x) {
     const int bb = b0 + tid;
-    int nA = 0, nB = 0, tF = 0, nF8 = 0, tF16 = 0;  // (tF, tF16: text tiles, each of hsg4 / hsg16 items)
+    int nA = 0, nB = 0, tF = 0, tF8 = 0, tF16 = 0;  // (tF..: text tiles, each of hsg4 / hsg16 items)
     if (bb < p.bt.B) {
       const int M = b0 == 0 ? M0 : (int)(p.bt.text_off[bb + 1] - p.bt.text_off[bb]);
       const int n1 = b0 == 0 ? n10 : *((volatile int32_t*)&p.n1[bb]);
@@ -76,7 +96,7 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
       if (fused4) {
         tF = (M + 127) / 128;
       } else if (fused8) {
-        nF8 = (M + 127) / 128;
+        tF8 = (M + 127) / 128;
       } else if (fused16) {
         tF16 = (M + 127) / 128;
       } else {
@@ -90,34 +110,36 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
         p.tau2[bb] = 0.f;
       }
     }
-    const int nS = tF * kFusedSlotsPerItem + nF8 * kFusedSlotsPerItem8 + tF16 * kFusedSlotsPerItem16 +
+    const int nS = tF * kFusedSlotsPerItem + tF8 * kFusedSlotsPerItem8 + tF16 * kFusedSlotsPerItem16 +
                    nB;  // s2(r) partial slots of this sample (a split tile's items share its slots)
-    const int nHS = hsg > 1 ? (hsC == 16 ? tF16 : tF) : 0;  // this sample's head-split tiles
-    // the seven item and slot counts, scanned together
-    __shared__ int mtmp[7 * 33];
-    const int cnt[7] = {nA, nB, tF * hsg4, nF8, tF16 * hsg16, nS, nHS};
-    int ex[7], tot[7];
-    block_exclusive_scan_n<7>(cnt, ex, tot, mtmp);
+    // this sample's head-split tiles, and the scratch slots of their items' CTAs
+    const int nHS = hsg > 1 ? (hs16 ? tF16 : tF + tF8) : 0;
+    const int hsC = hs16 ? 16 : tF ? kFusedCluster : 8;
+    // the eight item and slot counts, scanned together
+    __shared__ int mtmp[8 * 33];
+    const int cnt[8] = {nA, nB, tF * hsg4, tF8 * hsg4, tF16 * hsg16, nS, nHS, nHS * hsg * hsC};
+    int ex[8], tot[8];
+    block_exclusive_scan_n<8>(cnt, ex, tot, mtmp);
     const int totA = tot[0], totB = tot[1], totF = tot[2], totF8 = tot[3], totF16 = tot[4], totS = tot[5],
               totHS = tot[6];
     const int offA = runA + ex[0], offB = runB + ex[1], offF = runF + ex[2], offF8 = runF8 + ex[3],
-              offF16 = runF16 + ex[4], offS = runS + ex[5], offHS = runHS + ex[6];
+              offF16 = runF16 + ex[4], offS = runS + ex[5], offHS = runHS + ex[6], offP = runP + ex[7];
     if (bb < p.bt.B) {
       // a tile's items: one, or its head groups in turn
-      auto tile_items = [&](int4* items, int off, int tiles, int g_n, int slots) {
+      auto tile_items = [&](int4* items, int off, int tiles, int g_n, int C, int slots) {
         for (int t = 0; t < tiles; ++t)
           for (int g = 0; g < g_n; ++g, ++off)
             if (off < p.maxF)
-              items[off] = make_int4(bb, t * 128, offS + t * slots, g_n > 1 ? ((offHS + t) << 8) | (g << 4) | g_n : 0);
+              items[off] = make_int4(bb, t * 128, offS + t * slots,
+                                     g_n > 1 ? ((offP + (t * g_n + g) * C) << 8) | (g << 4) | g_n : 0);
       };
-      tile_items(p.itemsF, offF, tF, hsg4, kFusedSlotsPerItem);
-      tile_items(p.itemsF16, offF16, tF16, hsg16, kFusedSlotsPerItem16);
-      for (int i = 0; i < nF8; ++i)
-        if (offF8 + i < p.maxF) p.itemsF8[offF8 + i] = make_int4(bb, i * 128, offS + i * kFusedSlotsPerItem8, 0);
+      tile_items(p.itemsF, offF, tF, hsg4, kFusedCluster, kFusedSlotsPerItem);
+      tile_items(p.itemsF8, offF8, tF8, hsg4, 8, kFusedSlotsPerItem8);
+      tile_items(p.itemsF16, offF16, tF16, hsg16, 16, kFusedSlotsPerItem16);
       for (int t = 0; t < nHS; ++t)
         if (offHS + t < kHsMaxTiles)
-          p.itemsHS[offHS + t] = make_int4(
-              bb, t * 128, offS + t * (hsC == 16 ? kFusedSlotsPerItem16 : kFusedSlotsPerItem), hsg | (hsC << 8));
+          p.itemsHS[offHS + t] = make_int4(bb, t * 128, offS + t * hsC * kFusedPartialWarps,
+                                           hsg | (hsC << 8) | ((offP + t * hsg * hsC) << 16));
       p.itemA_off[bb] = offA;
       p.itemB_off[bb] = offB;
       p.slot_off[bb] = offS;
@@ -129,6 +151,7 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     runF16 += totF16;
     runS += totS;
     runHS += totHS;
+    runP += tot[7];
   }
   if (tid == 0) {
     p.itemA_off[p.bt.B] = runA;

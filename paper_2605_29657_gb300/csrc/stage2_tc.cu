@@ -118,7 +118,7 @@ namespace {
 
 struct ItemGeom {
   int b, j0, M, n, img0, own_img, txt0, own_txt, ip, tp, N, slot;
-  int h0, h1, nhg, hs_tile;  // heads [h0, h1) of this item; head groups of its tile (1: no split)
+  int h0, h1, nhg, hs_slot;  // heads [h0, h1) of this item; head groups of its tile (1: no split); its scratch slots
   bool fits;
   int64_t rbase, t0;
 };
@@ -154,7 +154,7 @@ __device__ __forceinline__ ItemGeom item_geom(const Stage2TcParams& p, int4 it, 
   g.nhg = hs_groups(it.w);
   g.h0 = hs_group(it.w) * p.H / g.nhg;
   g.h1 = (hs_group(it.w) + 1) * p.H / g.nhg;
-  g.hs_tile = hs_tile(it.w);
+  g.hs_slot = hs_slot(it.w);
   return g;
 }
 
@@ -707,8 +707,7 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
       if (g.nhg > 1) {
         // a head group of a split tile: its partial head sums go to the
         // scratch, rows of zeros past the text; the merge kernel reduces them
-        float* dst =
-            p.ppart + ((((int64_t)g.hs_tile * g.nhg + hs_group(p.items[item].w)) * C + rank) * kHsRows + j) * PMAX;
+        float* dst = p.ppart + ((int64_t)(g.hs_slot + rank) * kHsRows + j) * PMAX;
 #pragma unroll
         for (int q = 0; q < NPC; ++q) {
           if (q < npi) {
@@ -817,17 +816,47 @@ __global__ void __launch_bounds__(s2f::THREADS, 1)
   tc::cluster_sync_all();
 }
 
-// Merge of head-split tiles. CTA (t, rank) of a tiles x 16 grid takes tile t's S1 keys of cluster rank `rank`: key column k and row quarter q
-// belong to thread q * kFusedMaxOwnImg + k. A thread sums the head groups'
-// partials (in group order) for each of its rows (rows q, q + 4, ...), with
-// every load of its rows issued before the adds, and keeps their max and
-// sum; the four quarters then meet in shared memory in quarter order. The
-// column max over the tile's text rows goes to s2; the register columns'
-// sums over rows, added over the CTA's columns in a fixed order, fill the
-// tile's partial slots of that rank. The sample's last slot writer turns the
-// slots into ref2 and tau2 as the fused kernel does.
 constexpr int kMergeQ = 4;                            // row quarters per key column
 constexpr int kMergeThreads = kMergeQ * kFusedMaxOwnImg;
+// max and sum over a thread's rows q, q + 4, ... of the sums of nhg <= G head
+// groups' partials, 32 loads in flight at a time; sums in group order, then
+// row order
+template <int G>
+__device__ __forceinline__ void merge_rows(const float* src, uint32_t gstride, int nhg, int q, int rows, float& cmax,
+                                           float& rsum) {
+  constexpr int RU = 32 / G;
+  for (int r0 = q; r0 < rows; r0 += RU * kMergeQ) {
+    float v[RU][G];
+    uint32_t off = (uint32_t)r0 * s2f::PMAX;
+#pragma unroll
+    for (int hg = 0; hg < G; ++hg, off += gstride)
+#pragma unroll
+      for (int u = 0; u < RU; ++u)
+        v[u][hg] = (r0 + u * kMergeQ < rows && hg < nhg) ? __ldcg(src + (off + (uint32_t)(u * kMergeQ * s2f::PMAX))) : 0.f;
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+      if (r0 + u * kMergeQ < rows) {
+        float x = v[u][0];
+#pragma unroll
+        for (int hg = 1; hg < G; ++hg) x += v[u][hg];
+        cmax = fmaxf(cmax, x);
+        rsum += x;
+      }
+    }
+  }
+}
+
+// Merge of head-split tiles. CTA (t, rank) of a tiles x 16 grid takes tile t's
+// S1 keys of cluster rank `rank`: key column k and row quarter q belong to
+// thread q * kFusedMaxOwnImg + k. A thread sums the head groups' partials for
+// each of its rows (merge_rows) and keeps their max and sum; the four
+// quarters then meet in shared memory in quarter order. The column max over
+// the tile's text rows goes to s2; the register columns' sums over rows, added
+// over the CTA's columns in a fixed order, fill the tile's partial slots of
+// that rank. The sample's last slot writer turns the slots into ref2 and tau2
+// as the fused kernel does. Bound by its chain of memory round trips: 5 us
+// behind the fused kernel's end (8-10 with eight rows of eight groups loaded
+// at a time whatever the group count, which spilled).
 __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams p) {
   using namespace s2f;
   constexpr int NW = kFusedMaxOwnImg / 32;
@@ -837,17 +866,20 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
   const int t = blockIdx.x / 16, rank = blockIdx.x % 16;
   if (t >= p.counters[CNT_NHS]) return;
   const int4 it = p.itemsHS[t];
-  const int nhg = it.w & 255, C = it.w >> 8;
-  if (rank >= C) return;
-  const int4 whole = make_int4(it.x, it.y, it.z, 0);
-  const ItemGeom g = C == 16 ? item_geom<16>(p, whole, rank) : item_geom<kFusedCluster>(p, whole, rank);
+  const int nhg = it.w & 255, C = (it.w >> 8) & 255, slot0 = it.w >> 16;
+  // a launch behind the 8-CTA clusters takes their tiles, one behind the others the rest
+  if (rank >= C || (C == 8) != (p.merge8 != 0)) return;
+  // the tile's geometry, as item_geom has it
+  const int sb = it.x, j0 = it.y, slot = it.z;
+  const int M = (int)(p.bt.text_off[sb + 1] - p.bt.text_off[sb]), n = p.n1[sb];
+  const int per = (n + C - 1) / C, img0 = rank * per, own_img = max(0, min(per, n - img0));
   const int k = threadIdx.x % kFusedMaxOwnImg, q = threadIdx.x / kFusedMaxOwnImg, lane = threadIdx.x & 31;
-  const int rows = min(kHsRows, g.M - g.j0);
+  const int rows = min(kHsRows, M - j0);
   const float invH = 1.0f / (float)p.H;
   int row_id = 0;
   bool is_reg = false;
-  if (q == 0 && k < g.own_img) {
-    row_id = p.dense[g.rbase + g.img0 + k];
+  if (q == 0 && k < own_img) {
+    row_id = p.dense[p.bt.row_off[sb] + img0 + k];
     if (!in_bounds(row_id >= 0 && row_id < p.bt.total_rows, p.status, kSiteFusedKeyRow)) row_id = 0;
     is_reg = p.role[row_id] != 0;
   }
@@ -855,37 +887,22 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
   // kernel's partials (and its s2 and slot writes) only after it finished
   pdl_wait();
   float cmax = 0.f, rsum = 0.f;
-  if (k < g.own_img) {
-    const float* src = p.ppart + (((int64_t)t * nhg * C + rank) * kHsRows) * PMAX + k;
-    // this thread's rows q, q + 4, ..., up to eight at a time with every
-    // group's load in flight before the adds; sums in group order, then row
-    // order
-    for (int r0 = q; r0 < rows; r0 += 8 * kMergeQ) {
-      float v[8][kHsGroups];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-#pragma unroll
-        for (int hg = 0; hg < kHsGroups; ++hg) {
-          const int r = r0 + u * kMergeQ;
-          v[u][hg] = (r < rows && hg < nhg) ? __ldcg(src + ((int64_t)hg * C * kHsRows + r) * PMAX) : 0.f;
-        }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (r0 + u * kMergeQ < rows) {
-          float x = v[u][0];
-#pragma unroll
-          for (int hg = 1; hg < kHsGroups; ++hg) x += v[u][hg];
-          cmax = fmaxf(cmax, x);
-          rsum += x;
-        }
-      }
-    }
+  if (k < own_img) {
+    // 32-bit offsets: the scratch holds under 2^22 values
+    const float* src = p.ppart + (uint32_t)(slot0 + rank) * kHsRows * PMAX + k;
+    const uint32_t gstride = (uint32_t)C * kHsRows * PMAX;
+    if (nhg <= 2)
+      merge_rows<2>(src, gstride, nhg, q, rows, cmax, rsum);
+    else if (nhg <= 4)
+      merge_rows<4>(src, gstride, nhg, q, rows, cmax, rsum);
+    else
+      merge_rows<kHsGroups>(src, gstride, nhg, q, rows, cmax, rsum);
   }
   qpart[q][k] = make_float2(cmax, rsum);
   __syncthreads();
   float rc = 0.f;
   if (q == 0) {
-    if (k < g.own_img) {
+    if (k < own_img) {
       float cm = qpart[0][k].x, rs = qpart[0][k].y;
 #pragma unroll
       for (int qq = 1; qq < kMergeQ; ++qq) {
@@ -906,26 +923,26 @@ __global__ void __launch_bounds__(kMergeThreads) s2_merge_kernel(Stage2TcParams 
     float acc = 0.f;
     for (int w = 0; w < NW; ++w) acc += wsum[w];
     // the tile's NPW slots of this rank: the sum in the first, zeros after
-    p.refpart[g.slot + rank * NPW] = acc;
-    for (int i = 1; i < NPW; ++i) p.refpart[g.slot + rank * NPW + i] = 0.f;
+    p.refpart[slot + rank * NPW] = acc;
+    for (int i = 1; i < NPW; ++i) p.refpart[slot + rank * NPW + i] = 0.f;
     __threadfence();
-    const int nslots = p.slot_off[g.b + 1] - p.slot_off[g.b];
-    s_last = atomicAdd(&p.done[g.b], NPW) == nslots - NPW;
+    const int nslots = p.slot_off[sb + 1] - p.slot_off[sb];
+    s_last = atomicAdd(&p.done[sb], NPW) == nslots - NPW;
   }
   __syncthreads();
   if (s_last && threadIdx.x < 32) {
     // the sample's last partials: ref2 = (sum of the partials) / (R M),
     // lane l taking slots l, l + 32, ... in order, then a fixed tree
     __threadfence();
-    const int s0 = p.slot_off[g.b], s1 = p.slot_off[g.b + 1];
+    const int s0 = p.slot_off[sb], s1 = p.slot_off[sb + 1];
     float acc = 0.f;
     for (int i = s0 + lane; i < s1; i += 32) acc += __ldcg(&p.refpart[i]);
     acc = warp_sum_f(acc);
     if (lane == 0) {
-      const int R = p.bt.reg_off[p.bt.seg_first[g.b + 1]] - p.bt.reg_off[p.bt.seg_first[g.b]];
-      const float r2 = (R > 0 && g.M > 0) ? acc / ((float)R * (float)g.M) : 0.f;
-      p.ref2[g.b] = r2;
-      p.tau2[g.b] = p.lambda2 * r2;
+      const int R = p.bt.reg_off[p.bt.seg_first[sb + 1]] - p.bt.reg_off[p.bt.seg_first[sb]];
+      const float r2 = (R > 0 && M > 0) ? acc / ((float)R * (float)M) : 0.f;
+      p.ref2[sb] = r2;
+      p.tau2[sb] = p.lambda2 * r2;
     }
   }
 }

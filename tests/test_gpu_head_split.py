@@ -71,3 +71,13 @@ def test_split_equals_unsplit_route():
     # fp32 sums of 32 heads' probabilities in another grouping
     torch.testing.assert_close(torch.from_numpy(a["s2"]), torch.from_numpy(z["s2"]), rtol=4e-6, atol=1e-9)
     torch.testing.assert_close(torch.from_numpy(a["ref2"]), torch.from_numpy(z["ref2"]), rtol=4e-6, atol=1e-9)
+
+
+@pytest.mark.parametrize("P,M", [
+    ((900, 60, 400), (100, 130, 20)),                  # one sample on 8-CTA clusters beside two on 4
+    ((1533, 1000), (129, 250)),                        # all on 8-CTA clusters; 1,536 keys just fit
+    ((1534, 100), (20, 140)),                          # one that needs 16
+    ((800,) + (90,) * 7, (64,) * 8),
+])
+def test_split_with_larger_samples(P, M):
+    _check(P, M, seed=len(P) + P[0])
