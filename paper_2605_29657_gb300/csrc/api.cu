@@ -536,6 +536,12 @@ Stage2Params stage2_params(const occam_batch* b, const occam_stage2_args* a, con
     if (a->H2 % g == 0 && a->H2 / g >= 4 && (a->H2 / g) % (a->H2 / p.Hkv) == 0) p.hs_valid |= 1u << g;
   // (a split's CTAs need a slot each)
   p.res4 = widening_enabled() ? std::min(fused_resident_clusters(kFusedCluster), kHsSlots / kFusedCluster) : 0;
+  // (a tile count at most max_tiles, so at least this many groups fit)
+  const int most = p.res4 > 0 && max_tiles > 0 ? (int)std::min<int64_t>(p.res4 / max_tiles, kHsGroups) : 0;
+  p.sure4 = p.use_fused && p.has_ppart && (p.hs_valid & ((2u << most) - 1u)) != 0 &&
+                    fused_fits(kFusedCluster, b->max_sample_rows, b->max_text, a->H2)
+                ? 1
+                : 0;
   return p;
 }
 
@@ -603,10 +609,11 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     const int64_t max_tiles = (int64_t)b->B * cdiv(b->max_text, 128);
     const bool only16 = p.res16 > 0 && max_tiles <= p.res16 && (max_tiles == 1 || !q.ppart);
     const bool no2p = no_twopass(b, a);
-    // With the 16-CTA launch alone (one text tile) nothing runs beside it: no
-    // second stream, and it follows the finalize kernel with programmatic
-    // dependent launch.
-    const bool alone = only16 && no2p;
+    // With one launch alone (16 CTAs for one text tile, or 4 CTAs where the
+    // plan is sure to split the heads of samples that fit those) nothing runs
+    // beside it: no second stream, and it follows the finalize kernel with
+    // programmatic dependent launch.
+    const bool alone16 = only16 && no2p && !p.sure4, alone4 = p.sure4 != 0, alone = alone16 || alone4;
     q.pdl = 0;
     q.merge8 = 0;
     const int merge_tiles = (int)std::max<int64_t>(1, std::min<int64_t>(max_tiles, kHsMaxTiles));
@@ -627,7 +634,7 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     q8.items = p.itemsF8;
     q8.queue = p.counters + CNT_QUEUE8;
     const int ncl8 = fused_launch_clusters(8, L.maxF, sms);
-    if (p.split8) {
+    if (p.split8 && !alone) {
       if (launch_fused(8, mq, mk, mkt, q8, ncl8, beside) != 0) return OCCAM_ERR_CUDA;
       // head-split tiles (small batches) meet right behind the fused launches
       // of their stream
@@ -641,18 +648,19 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
     Stage2TcParams q16 = q;
     q16.items = p.itemsF16;
     q16.queue = p.counters + CNT_QUEUE16;
-    q16.pdl = alone && pdl ? 1 : 0;
+    q16.pdl = alone16 && pdl ? 1 : 0;
     const int ncl16 = fused_launch_clusters(16, L.maxF, sms);
-    if (launch_fused(16, mq, mk, mkt, q16, ncl16, st) != 0) return OCCAM_ERR_CUDA;
+    if (!alone4 && launch_fused(16, mq, mk, mkt, q16, ncl16, st) != 0) return OCCAM_ERR_CUDA;
     // the two-pass kernels (samples the fused kernel cannot hold; often none)
     // follow the 8-CTA launch on the second stream. They are enqueued after
     // the 16-CTA launch: a CTA of theirs takes a whole SM, and enqueued
     // earlier they held every SM before the 16-CTA clusters, which need 16
     // SMs of one GPC, could be placed.
-    if (!no2p) OCCAM_TRY(launch_twopass(p, L, sms, b, a, beside));
+    if (!no2p && !alone) OCCAM_TRY(launch_twopass(p, L, sms, b, a, beside));
     q.queue = p.counters + CNT_QUEUE4;
     const int ncl4 = fused_launch_clusters(4, L.maxF, sms);
-    if (!only16 && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
+    q.pdl = alone4 && pdl ? 1 : 0;
+    if ((!only16 || alone4) && launch_fused(4, mq, mk, mkt, q, ncl4, st) != 0) return OCCAM_ERR_CUDA;
     launch_s2_merge(q, merge_tiles, st);
     if (side) {
       OCCAM_CUDA(cudaEventRecord(side->join, side->stream));

@@ -123,6 +123,7 @@ struct Stage2Params {
   int4* itemsF16;           // fused items for 16-CTA clusters
   int use_fused;            // route eligible samples to the fused tensor-core kernel
   int res16, res8, res4;    // resident 16-, 8- and 4-CTA fused clusters (0: no widening or splitting for small batches)
+  int sure4;                // every sample fits 4-CTA clusters with all its rows in S1, and its heads split: the only launch
   int split8;               // the 8-CTA launch is made and may take split tiles
   uint32_t hs_valid;        // bit g: the heads split into g groups of whole key groups, at least 4 heads each
   int4* itemsHS;            // head-split text tiles (b, j0, slot, head groups | cluster size << 8 | first scratch slot << 16), for the merge kernel

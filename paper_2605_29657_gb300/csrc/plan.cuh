@@ -39,7 +39,7 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     if (p.has_ppart) {  // (at most kHsMaxTiles samples)
       if (tid < p.bt.B) {
         const bool fit4 = fused_fits(kFusedCluster, n10, M0, p.H);
-        fit = fit4 || (p.split8 && fused_fits(8, n10, M0, p.H));
+        fit = fit4 || (p.split8 && fused_fits(8, n10, M0, p.H)) || M0 == 0;
         tiles = min((M0 + 127) / 128, 100);
         tiles |= tiles * (fit4 ? kFusedCluster : 8) << 12;
       }
@@ -61,10 +61,13 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     // CTAs (36 resident) or 8 for the samples that do not fit those, take the
     // most groups: 8 tiles of 64 text rows and 540 S1 keys took 77 us on
     // 8-CTA clusters, a head after the other, and take 33 us and about 8 of
-    // merge in 4 groups. One tile has no use for that many, and more than
-    // kHsMaxTiles fill the device unsplit.
+    // merge in 4 groups; one tile of 32 text rows and 270 S1 keys 17 and 7 in
+    // 8 groups, where 16-CTA clusters in 4 groups take 21 and 7. (One tile
+    // does so only where the host can tell, p.sure4: else the launches for
+    // either would cost more than that.) More than kHsMaxTiles fill the device
+    // unsplit.
     if (p.has_ppart && total_tiles <= kHsMaxTiles) {
-      const bool small = __syncthreads_and(fit) && total_tiles > 1 && p.res4 > 0;
+      const bool small = __syncthreads_and(fit) && total_tiles > (p.sure4 ? 0 : 1) && p.res4 > 0;
       // the most groups that divide the heads (hs_valid) and fit at once
       int most = 0;
       if (small)

@@ -81,3 +81,14 @@ def test_split_equals_unsplit_route():
 ])
 def test_split_with_larger_samples(P, M):
     _check(P, M, seed=len(P) + P[0])
+
+
+@pytest.mark.parametrize("P,M,H2", [
+    ((576,), (32,), 32),                     # one tile, all rows fit 4-CTA clusters: that launch alone
+    ((40, 300, 700), (128, 5, 64), 32),
+    ((20, 30, 40, 50), (2, 130, 257, 4), 24),
+    ((60,), (20,), 6),                       # heads that do not split
+])
+def test_four_cta_launch_alone(P, M, H2):
+    _check(P, M, H2=H2, seed=sum(P))
+    _check(P, M, H2=H2, lam1=0.6, seed=sum(P))
