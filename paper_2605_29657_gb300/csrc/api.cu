@@ -115,6 +115,14 @@ BatchDev dev_batch(const occam_batch* b) {
   return d;
 }
 
+// Stage-I keys of more bytes than this (half of L2) pass through L2 marked to
+// leave it first: they are read once, and kept like other lines they pushed
+// out the rows the gather of the call before had just written, whose
+// write-back fell into the logits kernel (381 MB of keys: 79 us, 68 so; the
+// whole call 433.6 and 424.0). Fewer may stay for a caller that reads them
+// again.
+constexpr int64_t kL2StreamBytes = 64 << 20;
+
 int num_sms() {
   static int n = 0;
   static std::once_flag once;
@@ -363,6 +371,7 @@ int launch_stage1_scores(const occam_batch* b, const occam_stage1_args* a, const
     p.scale = (float)(1.4426950408889634 / std::sqrt((double)a->d1));  // logits in log2 units
     p.logits = at<float>(ws, L.stats1);
     p.status = status;
+    p.stream_keys = b->total_rows * a->H1 * a->d1 * 2 > kL2StreamBytes ? 1 : 0;
     const int64_t tiles = cdiv(b->total_rows, 16);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 2 * num_sms()));
     launch_stage1_logits(p, a->d1, grid, st);

@@ -55,6 +55,7 @@ struct Stage1ClsParams {
   const __nv_bfloat16* K1;
   float scale;  // log2(e) / sqrt(d1): [CLS] logits in log2 units
   float* logits;  // [rows, 16] per-head [CLS] logits in log2 units
+  int stream_keys;  // K1 passes through L2 without staying in it
   int* status;
 };
 

@@ -72,14 +72,23 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
   const int ntiles = (int)(nt_all * (blockIdx.x + 1) / gridDim.x - t0);
   const unsigned char* gsrc = reinterpret_cast<const unsigned char*>(p.K1);
 
+  // thread 0 issues the copies; keys too many to stay in L2 are marked to leave
+  // it first
+  const uint64_t policy = l2_evict_first();
+  auto load = [&](int st, int64_t r0, int rows) {
+    mbar_arrive_expect_tx(&bar[st], rows * kRowBytes);
+    if (p.stream_keys)
+      bulk_g2s_hint(smem + st * kStageBytes, gsrc + r0 * kRowBytes, rows * kRowBytes, &bar[st], policy);
+    else
+      bulk_g2s(smem + st * kStageBytes, gsrc + r0 * kRowBytes, rows * kRowBytes, &bar[st]);
+  };
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) mbar_init(&bar[i], 1);
     fence_mbar_init();
     for (int i = 0; i < kStages && i < ntiles; ++i) {
       const int64_t r0 = (t0 + i) * kTileRows;
       const int rows = (int)min((int64_t)kTileRows, R - r0);
-      mbar_arrive_expect_tx(&bar[i], rows * kRowBytes);
-      bulk_g2s(smem + i * kStageBytes, gsrc + r0 * kRowBytes, rows * kRowBytes, &bar[i]);
+      load(i, r0, rows);
     }
   }
   __syncthreads();
@@ -156,8 +165,7 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
     if (tid == 0 && it + kStages < ntiles) {
       const int64_t rn = (t0 + it + kStages) * kTileRows;
       const int rows_n = (int)min((int64_t)kTileRows, R - rn);
-      mbar_arrive_expect_tx(&bar[st], rows_n * kRowBytes);
-      bulk_g2s(smem + st * kStageBytes, gsrc + rn * kRowBytes, rows_n * kRowBytes, &bar[st]);
+      load(st, rn, rows_n);
     }
   }
   if (timed_out && tid == 0) {
