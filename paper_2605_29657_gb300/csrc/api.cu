@@ -719,18 +719,8 @@ int launch_compact(const occam_batch* b, const WsLayout& L, void* ws, int mode, 
     OCCAM_CUDA(cudaMemsetAsync(count_out, 0, b->B * 4, st));
     if (count_vis) OCCAM_CUDA(cudaMemsetAsync(count_vis, 0, b->B * 4, st));
   }
-  // without memsets just before it, the op ahead of the scan is a kernel that
-  // started after the call's counters were zeroed: programmatic dependent
-  // launch, the ticket and the row offsets read before that kernel finishes,
-  // everything else after (pdl_wait)
-  if (!do_memsets)
-    OCCAM_CUDA(launch_pdl(scan_kernel, dim3((unsigned)L.scan_tiles), dim3(256), 0, st, p));
-  else
-    scan_kernel<<<(unsigned)L.scan_tiles, 256, 0, st>>>(p);
-  count_launch();
-  trace.mark(st);
+  GatherParams g;
   if (n_tensors > 0) {
-    GatherParams g;
     g.n_tensors = n_tensors;
     for (int t = 0; t < OCCAM_MAX_GATHER; ++t) {
       g.src[t] = t < n_tensors ? static_cast<const unsigned char*>(src[t]) : nullptr;
@@ -743,6 +733,32 @@ int launch_compact(const occam_batch* b, const WsLayout& L, void* ws, int mode, 
     g.capacity = capacity;
     g.src_rows = b->total_rows;
     g.status = at<int>(ws, L.status);
+  }
+  // A batch of one scan tile: scan and gather in one launch (a traced call
+  // keeps them apart, for its intervals).
+  const bool one = L.scan_tiles == 1 && n_tensors > 0 && b->B <= kScanSmemSamples && !trace.ev;
+  // without memsets just before it, the op ahead of the scan is a kernel that
+  // started after the call's counters were zeroed: programmatic dependent
+  // launch, the ticket and the row offsets read before that kernel finishes,
+  // everything else after (pdl_wait)
+  if (one) {
+    // a warp per kept row and tensor, as far as the batch can have them
+    const int64_t warps = std::min<int64_t>(b->total_rows, std::max<int64_t>(capacity, 1)) * n_tensors;
+    const dim3 grid((unsigned)std::min<int64_t>(cdiv(warps, 8), (int64_t)num_sms() * 4));
+    if (!do_memsets)
+      OCCAM_CUDA(launch_pdl(compact_one_kernel, grid, dim3(256), 0, st, p, g));
+    else
+      compact_one_kernel<<<grid, 256, 0, st>>>(p, g);
+    count_launch();
+    return cuda_ok();
+  }
+  if (!do_memsets)
+    OCCAM_CUDA(launch_pdl(scan_kernel, dim3((unsigned)L.scan_tiles), dim3(256), 0, st, p));
+  else
+    scan_kernel<<<(unsigned)L.scan_tiles, 256, 0, st>>>(p);
+  count_launch();
+  trace.mark(st);
+  if (n_tensors > 0) {
     // programmatic dependent launch: scheduled as the scan ends, it waits for
     // the scan's results inside (pdl_wait)
     OCCAM_CUDA(launch_pdl(gather_kernel, dim3((unsigned)(num_sms() * 4)), dim3(256), 0, st, g));

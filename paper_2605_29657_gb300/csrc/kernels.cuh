@@ -339,7 +339,9 @@ int s2_fused_smem_bytes(int C);
 int s2_fused_threads();
 
 // compact.cu
+constexpr int kScanSmemSamples = 2048;  // samples whose offsets fit the scan's shared copy
 __global__ void scan_kernel(ScanParams p);
+__global__ void compact_one_kernel(ScanParams p, GatherParams g);
 __global__ void stage_rows_kernel(StageRowsParams p);
 __global__ void l2_keys_kernel(Lambda2Params p);
 __global__ void l2_hist_kernel(Lambda2Params p, int level);
