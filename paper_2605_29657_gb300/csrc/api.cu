@@ -358,7 +358,7 @@ struct Trace {
 // ---------------------------------------------------------------- launch helpers
 
 int launch_stage1_scores(const occam_batch* b, const occam_stage1_args* a, const WsLayout& L, void* ws,
-                         float* s1, float* s2_zero, cudaStream_t st, Trace trace = Trace()) {
+                         float* s1, float* s2_zero, cudaStream_t st, Trace trace = Trace(), bool zero = false) {
   const NvtxRange nvtx(a->mode == OCCAM_STAGE1_CLS ? "stage1_cls_scores" : "stage1_mutual_scores");
   const BatchDev bt = dev_batch(b);
   int* status = at<int>(ws, L.status);
@@ -372,6 +372,8 @@ int launch_stage1_scores(const occam_batch* b, const occam_stage1_args* a, const
     p.logits = at<float>(ws, L.stats1);
     p.status = status;
     p.stream_keys = b->total_rows * a->H1 * a->d1 * 2 > kL2StreamBytes ? 1 : 0;
+    p.zero = zero ? at<uint32_t>(ws, L.zero_begin) : nullptr;
+    p.zero_words = (int64_t)(L.zero_end - L.zero_begin) / 4;
     const int64_t tiles = cdiv(b->total_rows, 16);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 2 * num_sms()));
     launch_stage1_logits(p, a->d1, grid, st);
@@ -452,6 +454,7 @@ int launch_finalize1(const occam_batch* b, const WsLayout& L, void* ws, float* s
   p.n1_vis = n1_vis;
   p.seg_state = at<unsigned long long>(ws, L.seg_state);
   p.counters = at<int32_t>(ws, L.counters);
+  p.one_seg = b->S_tot == b->B ? 1 : 0;
   p.do_plan = plan ? 1 : 0;
   if (plan) p.plan = *plan;
   p.zero_count_out = count_out;
@@ -1029,9 +1032,13 @@ static int prune_impl(const occam_prune_args* args, const occam_prune_out* out, 
   int32_t* n1_vis = out->n1_vis ? out->n1_vis : at<int32_t>(ws, L.n1_vis);
   float* ref2 = out->ref2 ? out->ref2 : at<float>(ws, L.ref2);
   // every zero-initialised accumulator of the call, up front
-  OCCAM_CUDA(cudaMemsetAsync(at<unsigned char>(ws, L.zero_begin), 0, L.zero_end - L.zero_begin, st));
+  // (in the [CLS] logits kernel itself where the finalize kernel draws no
+  // segment ticket before it has waited for that kernel)
+  const bool zero_in_logits = args->stage1.mode == OCCAM_STAGE1_CLS && b->S_tot == b->B;
+  if (!zero_in_logits)
+    OCCAM_CUDA(cudaMemsetAsync(at<unsigned char>(ws, L.zero_begin), 0, L.zero_end - L.zero_begin, st));
   trace.mark(st);
-  OCCAM_TRY(launch_stage1_scores(b, &args->stage1, L, ws, s1, s2, st, trace));
+  OCCAM_TRY(launch_stage1_scores(b, &args->stage1, L, ws, s1, s2, st, trace, zero_in_logits));
   const Stage2Params plan = stage2_params(b, &a2, L, ws, s2, ref2, args->lambda2);
   OCCAM_TRY(launch_finalize1(b, L, ws, s1, nullptr, args->lambda1, 1, out->ref1, keep1, n1_vis, &args->stage1, s2,
                              &plan, out->count_out, out->count_vis, st, trace, out->n_eff,

@@ -56,6 +56,8 @@ struct Stage1ClsParams {
   float scale;  // log2(e) / sqrt(d1): [CLS] logits in log2 units
   float* logits;  // [rows, 16] per-head [CLS] logits in log2 units
   int stream_keys;  // K1 passes through L2 without staying in it
+  uint32_t* zero;   // nullable: words the first CTA zeroes (the call's accumulators)
+  int64_t zero_words;
   int* status;
 };
 
@@ -138,6 +140,7 @@ struct Stage2Params {
 };
 
 struct Stage1FinalizeParams {
+  int one_seg;  // one segment a sample: no look-back, so no segment ticket
   BatchDev bt;
   // [CLS] mode: the segment's s1 is first formed from the per-head logits
   // (softmax over the segment's rows and the [CLS] self key, head mean)

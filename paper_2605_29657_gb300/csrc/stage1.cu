@@ -72,6 +72,10 @@ __global__ void __launch_bounds__(cls::kThreads) stage1_logits_kernel(Stage1ClsP
   const int ntiles = (int)(nt_all * (blockIdx.x + 1) / gridDim.x - t0);
   const unsigned char* gsrc = reinterpret_cast<const unsigned char*>(p.K1);
 
+  // the call's accumulators, in place of a memset before this kernel (nothing
+  // touches them until the finalize kernel has waited for this one)
+  if (p.zero && blockIdx.x == 0)
+    for (int64_t i = tid; i < p.zero_words; i += kThreads) p.zero[i] = 0;
   // thread 0 issues the copies; keys too many to stay in L2 are marked to leave
   // it first
   const uint64_t policy = l2_evict_first();
@@ -347,8 +351,9 @@ __global__ void __launch_bounds__(256) stage1_finalize_kernel(Stage1FinalizePara
   __shared__ long long s_base;
   const int tid = threadIdx.x;
   // with S1 lists, segments are taken in ticket order: every earlier segment
-  // of the sample has started, so the look-back below always ends
-  if (tid == 0) s_seg = p.do_threshold ? atomicAdd(&p.counters[CNT_SEG_TICKET], 1) : (int)blockIdx.x;
+  // of the sample has started, so the look-back below always ends (a sample of
+  // one segment has none to look back to)
+  if (tid == 0) s_seg = p.do_threshold && !p.one_seg ? atomicAdd(&p.counters[CNT_SEG_TICKET], 1) : (int)blockIdx.x;
   __syncthreads();
   const int seg = s_seg;
   const int64_t sb = p.bt.seg_off[seg], se = p.bt.seg_off[seg + 1];
