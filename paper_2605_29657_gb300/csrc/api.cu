@@ -396,14 +396,23 @@ int launch_stage1_scores(const occam_batch* b, const occam_stage1_args* a, const
         !encode_map3(&mq1, a->q, b->total_rows, a->H1, a->d1, 16) ||
         !encode_map3(&mk1, a->K1, b->total_rows, a->H1, a->d1, 16))
       return OCCAM_ERR_CUDA;
-    p.tiles = (int)cdiv(b->max_seg_rows, kMutTileRows);
+    // CTA pairs from this many rows a segment on (on average; the host knows
+    // no more): 24,000 rows in segments of 904, 1,024 and 1,154 rows, 16 heads
+    // of 72, take 195, 173 and 232 us with one CTA an item and 198, 176 and
+    // 225 with pairs; 12 heads of 64 in segments of 644, 704 and 904 rows 155,
+    // 148 and 190 and 157, 146 and 182.
+    p.tile_rows = b->total_rows >= (a->d1 == 72 ? 1100 : 700) * (int64_t)b->S_tot ? kMutTileRows : 128;
+    p.tiles = (int)cdiv(b->max_seg_rows, p.tile_rows);
     // heads per item of the second pass: 4 (fewer item ends), less where the
     // batch would give a CTA pair under 12 items (at 6 images of 353-1,709
     // rows, 12 heads: 96 items of 4 heads for 76 pairs, whose longest pair
-    // gets 1.6 times the mean; 1.08 with one head each)
-    const int64_t mut_tiles = cdiv(b->total_rows, kMutTileRows) + b->S_tot / 2;
+    // gets 1.6 times the mean; 1.08 with one head each), or a CTA under 2
+    // (short items end often as it is: 24,000 rows in segments of 124, 12
+    // heads, 68 us in items of 4 heads and 76 of 2; 2,500 rows 29 and 27 of 1)
+    const int64_t mut_tiles = cdiv(b->total_rows, p.tile_rows) + b->S_tot / 2;
+    const int64_t wanted = (p.tile_rows == kMutTileRows ? 6 : 2) * (int64_t)num_sms();
     p.hgsize = 4;
-    while (p.hgsize > 1 && mut_tiles * cdiv(a->H1, p.hgsize) < 6 * (int64_t)num_sms()) p.hgsize >>= 1;
+    while (p.hgsize > 1 && mut_tiles * cdiv(a->H1, p.hgsize) < wanted) p.hgsize >>= 1;
     p.hgroups = (int)cdiv(a->H1, p.hgsize);
     p.part = p.lsum + (int64_t)a->H1 * b->total_rows;  // stats1 holds 2 * H1 floats per row
     p.queue = at<int32_t>(ws, L.counters) + CNT_MUT;

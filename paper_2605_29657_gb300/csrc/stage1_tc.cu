@@ -87,11 +87,6 @@ struct Cfg {
   static constexpr bool FOLD = PASS == 2 && D == 72;
   static constexpr bool LSM = PASS == 2 && !FOLD;  // the softmax warps take the log-sums from shared memory
   static constexpr int NBB = LSM && T1 ? 6 : 8;     // half blocks of B in flight (a ring; A tiles and accumulators: 2 each)
-  // The tensor core truncates its fp32 sums, which pulls S - L / c toward zero
-  // and every probability up alike; -L / c is given that much more. The
-  // 2-norm error of s1 against 64 bits, on segments of 100-4,000 rows, is
-  // 0.7e-7-1.0e-7 with it and 7e-7-11e-7 without.
-  static constexpr float kFoldBias = 0.94f * 5.9604644775390625e-08f;  // times 2^-24
 };
 
 template <int PASS, int D>
@@ -551,7 +546,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(m1::THREADS, 1)
             const float r1 = y - __bfloat162float(h1);
             const __nv_bfloat16 h2 = __float2bfloat16_rn(r1);
             const float r2 = r1 - __bfloat162float(h2);
-            const __nv_bfloat16 h3 = __float2bfloat16_rn(fmaf(y, CF::kFoldBias, r2));
+            const __nv_bfloat16 h3 = __float2bfloat16_rn(fmaf(y, kMutFoldBias, r2));
             t4.x = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
             t4.y = (uint32_t)__bfloat16_as_ushort(h3);
           }
@@ -784,20 +779,23 @@ void launch_passes(const MutualTcParams& p, const CUtensorMap& mq, const CUtenso
   mutual_tc_kernel<1, D><<<grid, m1::THREADS, smem1, st>>>(mq, mk, mq1, mk1, p);
   mutual_tc_kernel<1, D, true><<<grid, m1::THREADS, smem1, st>>>(mq, mk, mq1, mk1, p);
   mutual_tc_kernel<2, D><<<grid, m1::THREADS, smem2, st>>>(mk, mq, mk1, mq1, p);
+  count_launch(3);
 }
 }  // namespace
 
 void launch_mutual_tc(const MutualTcParams& p, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mq1,
                       const CUtensorMap& mk1, int sms, cudaStream_t st) {
   const int grid = std::max(2, sms & ~1);  // CTA pairs
-  if (p.d1 == 64)
+  if (p.tile_rows != kMutTileRows)
+    launch_mutual_short(p, mq, mk, mq1, mk1, sms, st);
+  else if (p.d1 == 64)
     launch_passes<64>(p, mq, mk, mq1, mk1, grid, st);
   else if (p.d1 == 72)
     launch_passes<72>(p, mq, mk, mq1, mk1, grid, st);
   else
     launch_passes<80>(p, mq, mk, mq1, mk1, grid, st);
   mutual_reduce_kernel<<<sms * 2, 256, 0, st>>>(p);
-  count_launch(4);
+  count_launch();
 }
 
 }  // namespace occam

@@ -1,7 +1,8 @@
-"""Mutual Stage I on CTA pairs, at the edges of its tiles (256 rows an item,
-128 a CTA, blocks of 256 keys taken in turn by two groups of softmax warps),
-with head counts that leave a ragged head group, and with logits that overflow
-the first pass's running sums (items worked through a second time)."""
+"""Mutual Stage I on CTA pairs (batches of long segments on average) and on
+single CTAs (short ones), at the edges of their tiles (256 rows an item, 128 a
+CTA, blocks of 256 keys taken in turn by two groups of softmax warps), with
+head counts that leave a ragged head group, and with logits that overflow the
+pairs' first pass's running sums (items worked through a second time)."""
 
 from __future__ import annotations
 
@@ -55,13 +56,16 @@ def _check(rows, H, d, seed, scale=None, rtol=4e-6, plain=False):
 @pytest.mark.parametrize("d", [64, 72, 80])
 @pytest.mark.parametrize("H", [1, 3, 16])
 def test_tile_edges(d, H):
-    _check([2, 127, 128, 129, 255, 256, 257, 384, 385, 511, 513, 769], H, d, seed=d + H)
+    edges = [2, 127, 128, 129, 255, 256, 257, 384, 385, 511, 513, 769]
+    _check(edges, H, d, seed=d + H)
+    # two long segments bring the mean past the line to the pairs
+    _check([5900] + edges + [6000], H, d, seed=d + H, plain=True)
 
 
 @pytest.mark.parametrize("d,H", [(72, 10), (64, 6)])
 def test_head_groups_of_a_larger_batch(d, H):
     """Enough tiles for items of four heads, with a ragged last group."""
-    _check([1100, 900, 1300, 700] * (20 if H > 8 else 30), H, d, seed=7, plain=True)
+    _check([1500, 1100, 1300, 900] * (20 if H > 8 else 30), H, d, seed=7, plain=True)
 
 
 @pytest.mark.parametrize("d", [64, 72, 80])
@@ -77,4 +81,5 @@ def test_overflowing_sums_are_redone(d):
         f[off[2] + 300:off[3]] = 128
         return torch.from_numpy(f)
 
-    _check([600, 300, 700], 4, d, seed=d, scale=scale, rtol=1e-3)
+    _check([1500, 900, 1300], 4, d, seed=d, scale=scale, rtol=1e-3)
+    _check([600, 300, 700], 4, d, seed=d, scale=scale, rtol=1e-3)  # (single CTAs)
