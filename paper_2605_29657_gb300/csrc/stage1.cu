@@ -351,9 +351,19 @@ __global__ void __launch_bounds__(256) stage1_finalize_kernel(Stage1FinalizePara
   __shared__ long long s_base;
   const int tid = threadIdx.x;
   // with S1 lists, segments are taken in ticket order: every earlier segment
-  // of the sample has started, so the look-back below always ends (a sample of
-  // one segment has none to look back to)
-  if (tid == 0) s_seg = p.do_threshold && !p.one_seg ? atomicAdd(&p.counters[CNT_SEG_TICKET], 1) : (int)blockIdx.x;
+  // of the sample has started, so the look-back below always ends. A sample of
+  // one segment has none to look back to: where all samples are such (as many
+  // segments as samples says so unless a sample has no rows) the block's index
+  // does. The counters may then be zeroed by the kernel ahead, which a ticket
+  // waits for.
+  bool ticket = p.do_threshold;
+  if (ticket && p.one_seg) {
+    bool same = true;
+    for (int i = tid; i < p.bt.B; i += blockDim.x) same &= p.bt.seg_first[i] == i;
+    ticket = !__syncthreads_and(same);
+    if (ticket) pdl_wait();
+  }
+  if (tid == 0) s_seg = ticket ? atomicAdd(&p.counters[CNT_SEG_TICKET], 1) : (int)blockIdx.x;
   __syncthreads();
   const int seg = s_seg;
   const int64_t sb = p.bt.seg_off[seg], se = p.bt.seg_off[seg + 1];

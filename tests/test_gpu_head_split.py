@@ -92,3 +92,36 @@ def test_split_with_larger_samples(P, M):
 def test_four_cta_launch_alone(P, M, H2):
     _check(P, M, H2=H2, seed=sum(P))
     _check(P, M, H2=H2, lam1=0.6, seed=sum(P))
+
+
+def test_as_many_segments_as_samples_with_one_sample_empty():
+    """Two samples of two segments between two without a row: their S1 lists
+    still follow the order of their segments."""
+    P, M = (60, 200), (40, 30)
+    b = tiny_batch(B=2, segs=2, P=P, R=2, M=M, H1=16, d1=64, H2=32, d2=128, hidden=64, seed=3, beta1=2.0)
+    want = run_prune(b, 0.2, 1.0)
+    m = dict(b["meta"])
+    r = m["row_off_host"]
+    # the last text token of each sample becomes a rowless sample's
+    m["row_off_host"] = torch.tensor([0, r[1], r[1], r[2], r[2]]).numpy()
+    m["text_off_host"] = torch.tensor([0, 39, 40, 69, 70]).numpy()
+    got = run_prune(dict(b, meta=m), 0.2, 1.0)
+    assert got["status"] == 0 == want["status"]
+    for k in ("s1", "ref1", "keep1"):
+        assert (got[k] == want[k]).all(), k
+    assert got["n1_vis"][0::2].tolist() == want["n1_vis"].tolist()
+    # the same samples with that text alone, each a batch of its own
+    assert got["count_out"][1::2].tolist() == [0, 0]
+    o = got["out_off"]
+    assert (o[1::2] == o[2::2]).all() and o[4] == got["count_out"].sum()
+    keep2 = got["keep2"].nonzero()[0]
+    assert got["out_index"][:o[4]].tolist() == keep2.tolist()
+    one = dict(b)
+    m1 = dict(b["meta"])
+    keep = [i for i in range(70) if i not in (39, 69)]
+    one["Q_text"], one["K_text"] = b["Q_text"][keep], b["K_text"][keep]
+    m1["text_off_host"] = torch.tensor([0, 39, 68]).numpy()
+    one["meta"] = m1
+    z = run_prune(one, 0.2, 1.0)
+    # fp32 sums of 32 heads' probabilities in another grouping
+    torch.testing.assert_close(torch.from_numpy(got["s2"]), torch.from_numpy(z["s2"]), rtol=4e-6, atol=1e-9)
