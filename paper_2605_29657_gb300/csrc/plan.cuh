@@ -128,17 +128,21 @@ __device__ __forceinline__ void plan_stage2(const Stage2Params& p, int* tmp) {
     const int offA = runA + ex[0], offB = runB + ex[1], offF = runF + ex[2], offF8 = runF8 + ex[3],
               offF16 = runF16 + ex[4], offS = runS + ex[5], offHS = runHS + ex[6], offP = runP + ex[7];
     if (bb < p.bt.B) {
-      // a tile's items: one, or its head groups in turn
-      auto tile_items = [&](int4* items, int off, int tiles, int g_n, int C, int slots) {
-        for (int t = 0; t < tiles; ++t)
-          for (int g = 0; g < g_n; ++g, ++off)
-            if (off < p.maxF)
-              items[off] = make_int4(bb, t * 128, offS + t * slots,
-                                     g_n > 1 ? ((offP + (t * g_n + g) * C) << 8) | (g << 4) | g_n : 0);
-      };
-      tile_items(p.itemsF, offF, tF, hsg4, kFusedCluster, kFusedSlotsPerItem);
-      tile_items(p.itemsF8, offF8, tF8, hsg4, 8, kFusedSlotsPerItem8);
-      tile_items(p.itemsF16, offF16, tF16, hsg16, 16, kFusedSlotsPerItem16);
+      // the sample's tiles, all on clusters of one size; a tile's items: one, or
+      // its head groups in turn (one rolled loop: this code runs once a call, on
+      // one CTA, and waits for its instructions)
+      int4* const items = tF ? p.itemsF : tF8 ? p.itemsF8 : p.itemsF16;
+      const int C = tF ? kFusedCluster : tF8 ? 8 : 16, g_n = tF16 ? hsg16 : hsg4;
+      const int tiles = tF + tF8 + tF16, slots = C * kFusedPartialWarps;
+      int off = tF ? offF : tF8 ? offF8 : offF16;
+#pragma unroll 1
+      for (int t = 0; t < tiles; ++t)
+#pragma unroll 1
+        for (int g = 0; g < g_n; ++g, ++off)
+          if (off < p.maxF)
+            items[off] = make_int4(bb, t * 128, offS + t * slots,
+                                   g_n > 1 ? ((offP + (t * g_n + g) * C) << 8) | (g << 4) | g_n : 0);
+#pragma unroll 1
       for (int t = 0; t < nHS; ++t)
         if (offHS + t < kHsMaxTiles)
           p.itemsHS[offHS + t] = make_int4(bb, t * 128, offS + t * hsC * kFusedPartialWarps,
