@@ -697,6 +697,15 @@ int launch_stage2(const occam_batch* b, const occam_stage2_args* a, const WsLayo
   return cuda_ok();
 }
 
+// The mean reference of n units of at most max_rows rows each.
+void launch_mean_ref(const MeanRefParams& p, int n, int64_t max_rows, cudaStream_t st) {
+  if (max_rows > kMeanSplitRows)
+    mean_ref_split_kernel<<<(unsigned)n * 8u, 256, 0, st>>>(p);
+  else
+    mean_ref_kernel<<<n, 256, 0, st>>>(p);
+  count_launch();
+}
+
 int launch_compact(const occam_batch* b, const WsLayout& L, void* ws, int mode, const uint8_t* keep_in,
                    const uint8_t* keep1, const float* s2, int keep_registers, uint8_t* keep_out, int n_tensors,
                    const void* const* src, const int64_t* row_bytes, void* const* dst, int64_t capacity,
@@ -891,8 +900,8 @@ int occam_mean_reference(const occam_batch* batch, const float* s, int32_t ref_s
   p.ref = ref;
   p.lambda = 0.f;
   p.tau = nullptr;
-  mean_ref_kernel<<<ref_scope == OCCAM_REF_SEGMENT ? batch->S_tot : batch->B, 256, 0, st>>>(p);
-  count_launch();
+  launch_mean_ref(p, ref_scope == OCCAM_REF_SEGMENT ? batch->S_tot : batch->B,
+                  ref_scope == OCCAM_REF_SEGMENT ? batch->max_seg_rows : batch->max_sample_rows, st);
   return cuda_ok();
 }
 
@@ -1101,8 +1110,7 @@ static int prune_impl(const occam_prune_args* args, const occam_prune_out* out, 
     mp.ref = ref2;
     mp.lambda = args->lambda2;
     mp.tau = at<float>(ws, L.tau2);
-    mean_ref_kernel<<<b->B, 256, 0, st>>>(mp);
-    count_launch();
+    launch_mean_ref(mp, b->B, b->max_sample_rows, st);
     OCCAM_CUDA(cudaGetLastError());
   }
   return launch_compact(b, L, ws, 1, nullptr, keep1, s2, args->keep_registers, out->keep2, args->n_tensors,

@@ -364,7 +364,9 @@ __global__ void registers_kernel(RegistersParams p);
 int launch_l2_cluster(const Lambda2Params& p, cudaStream_t st);
 
 // rules.cu
+constexpr int kMeanSplitRows = 2048;  // units of more rows are summed by 8 CTAs each
 __global__ void mean_ref_kernel(MeanRefParams p);
+__global__ void mean_ref_split_kernel(MeanRefParams p);
 int launch_budget_keep(const BudgetParams& p, int64_t max_sample_rows, cudaStream_t st);
 __global__ void pool_scores_kernel(const float* s_in, int64_t rows_out, int group, int mode, float* s_out);
 __global__ void gather_kernel(GatherParams p);

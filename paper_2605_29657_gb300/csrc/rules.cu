@@ -14,6 +14,8 @@
 //                       group of consecutive rows.
 // All are deterministic: fixed-order sums, and a selection whose result
 // does not depend on thread timing.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -25,14 +27,21 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// One CTA of 256 threads per unit (segment or sample). Thread t sums the
-// candidate rows t, t + 256, ... in fp64; warps then combine in a fixed tree
-// and warp 0's lane 0 adds the eight warp sums in order.
-__global__ void __launch_bounds__(256) mean_ref_kernel(MeanRefParams p) {
-  __shared__ double wsum[8];
-  __shared__ int wcnt[8];
+// A cluster of C CTAs of 256 threads per unit (segment or sample). Thread t of
+// CTA c sums the candidate rows 256 c + t, 256 (c + C) + t, ... in fp64; warps
+// then combine in a fixed tree, a CTA's lane 0 adds its eight warp sums in
+// order and the first CTA's the C sums. What bounds it is the rounds of loads
+// and the slow fp64 adds of one SM, so units of more than kMeanSplitRows rows
+// take eight CTAs: 5 samples of 3,500 to 14,900 rows 31.3 us with one CTA each
+// and a row a round, 6.2 so; 64 samples of 2,900 rows 17.0 and 8.2. Below, the
+// rounds of four rows alone: 21 samples of 420 to 890 rows 5.9 and 4.0.
+template <int C>
+__device__ __forceinline__ void mean_ref(const MeanRefParams& p) {
+  constexpr int PER = 4;
+  __shared__ double wsum[8], csum[C];
+  __shared__ int wcnt[8], ccnt[C];
   __shared__ uint32_t bits[kRegBitWords];
-  const int u = blockIdx.x, tid = threadIdx.x;
+  const int u = blockIdx.x / C, rank = blockIdx.x % C, tid = threadIdx.x;
   const int64_t lo = p.scope == OCCAM_REF_SEGMENT ? p.bt.seg_off[u] : p.bt.row_off[u];
   const int64_t hi = p.scope == OCCAM_REF_SEGMENT ? p.bt.seg_off[u + 1] : p.bt.row_off[u + 1];
   if (!p.role) {
@@ -43,10 +52,25 @@ __global__ void __launch_bounds__(256) mean_ref_kernel(MeanRefParams p) {
   }
   double acc = 0.0;
   int cnt = 0;
-  for (int64_t r = lo + tid; r < hi; r += blockDim.x) {
-    if (!(p.role ? p.role[r] != 0 : test_bit(bits, (int)(r - lo))) && (!p.prev_keep || p.prev_keep[r] != 0)) {
-      acc += (double)p.s[r];
-      ++cnt;
+  // PER rows' loads are in flight together
+  for (int64_t r0 = lo + rank * 256 + tid; r0 < hi; r0 += PER * C * 256) {
+    float s[PER];
+    bool cand[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      const int64_t r = r0 + k * C * 256;
+      const bool in = r < hi;
+      s[k] = in ? p.s[r] : 0.f;
+      const bool kept = in && (!p.prev_keep || p.prev_keep[r] != 0);
+      const bool reg = in && p.role && p.role[r] != 0;
+      cand[k] = kept && !reg;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      if (cand[k] && (p.role || !test_bit(bits, (int)(r0 - lo) + k * C * 256))) {
+        acc += (double)s[k];
+        ++cnt;
+      }
     }
   }
   acc = warp_sum_d(acc);
@@ -56,18 +80,41 @@ __global__ void __launch_bounds__(256) mean_ref_kernel(MeanRefParams p) {
     wcnt[tid >> 5] = cnt;
   }
   __syncthreads();
-  if (tid == 0) {
-    double a = 0.0;
-    int c = 0;
+  double a = 0.0;
+  int c = 0;
+  if (tid == 0)
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
       a += wsum[w];
       c += wcnt[w];
     }
+  if constexpr (C > 1) {
+    // every CTA runs, then every sum is in the first one's shared memory
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (tid == 0) {
+      cl.map_shared_rank(csum, 0)[rank] = a;
+      cl.map_shared_rank(ccnt, 0)[rank] = c;
+    }
+    cl.sync();
+    if (rank != 0) return;
+    if (tid == 0) {
+      a = 0.0;
+      c = 0;
+      for (int i = 0; i < C; ++i) {
+        a += csum[i];
+        c += ccnt[i];
+      }
+    }
+  }
+  if (tid == 0) {
     const float ref = c > 0 ? (float)(a / (double)c) : 0.f;
     p.ref[u] = ref;
     if (p.tau) p.tau[u] = p.lambda * ref;
   }
 }
+__global__ void __launch_bounds__(256) mean_ref_kernel(MeanRefParams p) { mean_ref<1>(p); }
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(256) mean_ref_split_kernel(MeanRefParams p) { mean_ref<8>(p); }
 
 // Order-preserving 32-bit key of a float: larger values give larger keys
 // (-0 is taken as +0, so equal values have equal keys; NaN is undefined).

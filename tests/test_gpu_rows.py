@@ -137,3 +137,18 @@ def test_calibrate_lambda2_row_ranges(seg_rows, segs):
             lam, got = occ.occam_calibrate_lambda2(lay, *args, K)
             assert int(got[0]) == cnt == nc
             assert np.float32(lam[0].item()) == want, (K, spread, tiny)
+
+
+@pytest.mark.parametrize("rows", [[2048, 5], [2049, 1, 255, 257, 300], [16385, 2304, 1]])
+def test_mean_reference_at_the_split(rows):
+    """Units summed by one CTA (2,048 rows at most) and by eight."""
+    import paper_2605_29657_gb300 as occ
+
+    lay, seg_off, _, is_reg, rng = _layout(rows, [1] * len(rows), 1, seed=len(rows))
+    n = int(seg_off[-1])
+    s = rng.integers(0, 200, n).astype(np.float32) / 16
+    pk = (rng.random(n) < 0.5).astype(np.uint8)
+    for scope in (occ.OCCAM_REF_SEGMENT, occ.OCCAM_REF_SAMPLE):
+        ref = occ.occam_mean_reference(lay, torch.from_numpy(s).cuda(), scope, prev_keep=torch.from_numpy(pk).cuda())
+        # sums of multiples of 1/16 are exact in fp64 in any order
+        assert (ref.cpu().numpy() == O.mean_reference(s, seg_off, ~is_reg & pk.astype(bool)).astype(np.float32)).all()
