@@ -119,8 +119,9 @@ BatchDev dev_batch(const occam_batch* b) {
 // leave it first: they are read once, and kept like other lines they pushed
 // out the rows the gather of the call before had just written, whose
 // write-back fell into the logits kernel (381 MB of keys: 79 us, 68 so; the
-// whole call 433.6 and 424.0). Fewer may stay for a caller that reads them
-// again.
+// whole call 433.6 and 424.0; Stage I on 73, 89 and 110 MB 27.3, 36.9 and 33.2
+// us, and 25.9, 35.2 and 31.0 so). Fewer may stay for a caller that reads them
+// again at once (89 MB of keys that L2 still holds: 31 us, marked 35).
 constexpr int64_t kL2StreamBytes = 64 << 20;
 
 int num_sms() {
